@@ -395,9 +395,7 @@ int hamr_grid_create(const hamr_grid_desc* d, hamr_grid** out) {
     g->desc = *d;
     g->blocks.assign(d->blocks, d->blocks + d->nblocks);
     g->desc.blocks = g->blocks.data();
-    g->ph.gam = d->gam;
-    g->ph.igam = 1.0 / d->gam;
-    g->ph.gfac = (d->gam - 1.0) * g->ph.igam;
+    set_gam(g->ph, d->gam);
     g->ph.cour = d->cour;
     g->ph.recon = d->recon;
     g->ph.riemann = d->riemann;
