@@ -13,6 +13,7 @@
 // in [0, 1 - 1/50^2].
 #pragma once
 #include "../../include/hamr.h"
+#include "ff.cuh"
 #include "grmhd.cuh"
 
 namespace hamr {
@@ -93,6 +94,120 @@ __device__ __forceinline__ bool newton_wv(const C2PScalars& S, double gfac, doub
     return ok;
 }
 
+// newton_wv out of line, for the callers below whose common path it is not (its registers and code
+// stay out of theirs)
+struct NewtonOut {
+    double W, vsq;
+    int it;
+    bool ok;
+};
+static __device__ __noinline__ NewtonOut newton_wv_call(const C2PScalars* S, double gfac, double W, double vsq) {
+    NewtonOut o;
+    o.ok = newton_wv(*S, gfac, W, vsq, o.it);
+    o.W = W;
+    o.vsq = vsq;
+    return o;
+}
+
+// newton_wv with its iterations in double-float (ff.cuh) and the last word from FP64: the same
+// iterations, from the same start to the same stopping rule, on the equations scaled by the power of two
+// that brings the start's W to [1, 2) (f1 ~ W, f2 ~ W^2), on the FP32 pipe; then the FP64 residuals at
+// that root, solved with the Jacobian of the last iteration. The double-float root is 1e-13 or better, so
+// that solve (relative error of the Jacobian 1e-7 times its cancellation) leaves what FP64 residuals
+// resolve, like newton_wv's own last iterate. Taken when the step and the step times the cancellation
+// (|j11 j22| + |j12 j21|) / |det| are as small as that argument needs; otherwise, and wherever the
+// double-float iteration meets no root or leaves its range, newton_wv decides. `it` counts the iterations,
+// not the solve. rs: 1/sqrt(1 - v^2) at the root where it comes for free, else 0.
+// An FP64 iteration is ~52 FP64 instructions (64 cycles each per scheduler), here ~340 FP32 ones, plus
+// ~28 FP64 for the solve: 1,000,003 states from a 5% start (4.7 iterations) 1021 -> 564 us with the entropy
+// backup below, the FP64 cell update of the 256x128x64 torus 2.00 -> 1.50 ms.
+__device__ __forceinline__ bool newton_wv_ff(const C2PScalars& S, double gfac, double& W, double& vsq, int& it,
+                                             double& rs64) {
+    rs64 = 0.0;
+    const unsigned eW = (unsigned)__double2hiint(W) & 0xfff00000u;  // sign and exponent of the start
+    bool ok = false;
+    if (eW - 0x2b000000u < 0x2a000000u) {  // W positive, 2^-334 .. 2^337
+        const unsigned sh = 0x3ff00000u - eW;
+        const ff D = ff_of(S.D, (int)sh), B2 = ff_of(S.Bsq, (int)sh), Qn = ff_of(S.Qdotn, (int)sh);
+        const ff Qt = ff_of(S.Qtsq, (int)(2u * sh)), QB = ff_of(S.QB2, (int)(3u * sh));
+        const ff gf = ff_of(gfac), one{1.0f, 0.0f};
+        const ff vmax{(float)C2P_VSQMAX, (float)(C2P_VSQMAX - (double)(float)C2P_VSQMAX)};
+        const ff hB = ff_scale(B2, 0.5f), c1 = ff_neg(ff_add(hB, Qn));
+        ff w = ff_of(W, (int)sh), v = ff_of(vsq);
+        float j11h = 0.0f, j12h = 0.0f, j21h = 0.0f, j22h = 0.0f, idh = 0.0f, iwh = 0.0f, rsh = 0.0f;
+        for (it = 1; it <= C2P_NMAX; it++) {
+            const ff omv = ff_sub(one, v);
+            const ff rs = ff_rsqrt(omv);
+            const ff bw = ff_add(B2, w);
+            const ff p = ff_mul(gf, ff_sub(ff_mul(w, omv), ff_mul(D, ff_mul(omv, rs))));
+            const ff iw = ff_rcp(w);
+            const ff q2 = ff_mul(QB, ff_mul(iw, iw)), q3 = ff_mul(q2, iw);
+            const ff j22 = ff_mul(bw, bw);
+            // f1 = -B^2 (1 + v)/2 + QB2/(2 W^2) - W + p - Q.n, f2 = v (B^2 + W)^2 - QB2 (B^2 + 2 W)/W^2 - Qt^2
+            const ff f1 = ff_add(ff_sub(ff_sub(ff_scale(q2, 0.5f), w), ff_mul(hB, v)), ff_add(p, c1));
+            const ff f2 = ff_sub(ff_sub(ff_mul(v, j22), Qt), ff_mul(q2, ff_add(bw, w)));
+            const ff j11 = ff_sub(ff_sub(ff_mul(gf, omv), one), q3);
+            const ff j12 = ff_sub(ff_mul(gf, ff_sub(ff_scale(ff_mul(D, rs), 0.5f), w)), hB);
+            const ff j21 = ff_scale(ff_mul(bw, ff_add(v, q3)), 2.0f);
+            const ff id = ff_rcp(ff_sub(ff_mul(j11, j22), ff_mul(j12, j21)));
+            const ff dw = ff_mul(ff_sub(ff_mul(j12, f2), ff_mul(j22, f1)), id);
+            const ff dv = ff_mul(ff_sub(ff_mul(j21, f1), ff_mul(j11, f2)), id);
+            const ff wn = ff_add(w, dw);
+            ff vn = ff_add(v, dv);
+            if (vn.h < 0.0f) vn = ff{0.0f, 0.0f};
+            if (!ff_less(vn, vmax)) vn = vmax;
+            if (!(wn.h > 0.0f && wn.h < 1e9f)) break;  // NaNs too
+            const float err = fabsf(dw.h) + fabsf((vn.h - v.h) + (vn.l - v.l)) * wn.h;
+            w = wn;
+            v = vn;
+            if (err < (float)C2P_TOL * wn.h) {
+                ok = true;
+                j11h = j11.h;
+                j12h = j12.h;
+                j21h = j21.h;
+                j22h = j22.h;
+                idh = id.h;
+                iwh = iw.h;
+                rsh = rs.h;
+                break;
+            }
+        }
+        if (ok) {
+            double Wd = ff_d(w);  // in [2^-40, 2^30]: the exponent added back as an integer
+            Wd = __hiloint2double((int)((unsigned)__double2hiint(Wd) - sh), __double2loint(Wd));
+            const double vd = ff_d(v);
+            const double omv = 1.0 - vd;
+            const double r = rsqrt(omv);
+            const double W2 = Wd * Wd, BW = S.Bsq + Wd;
+            const double p = gfac * (Wd * omv - S.D * (omv * r));
+            const double f1 = (-0.5 * S.Bsq * (1.0 + vd) - Wd + p - S.Qdotn) * W2 + 0.5 * S.QB2;
+            const double f2 = (vd * BW * BW - S.Qtsq) * W2 - S.QB2 * (BW + Wd);
+            const float iw2 = iwh * iwh;
+            const float r1 = ff_of(f1, (int)(3u * sh)).h * iw2, r2 = ff_of(f2, (int)(4u * sh)).h * iw2;
+            const float dw = (j12h * r2 - j22h * r1) * idh, dv = (j21h * r1 - j11h * r2) * idh;
+            const float step = fabsf(dw) + fabsf(dv) * w.h;
+            const float cancel = (fabsf(j11h * j22h) + fabsf(j12h * j21h)) * fabsf(idh);
+            const double vn = vd + widen(dv);
+            const long long vb = __double_as_longlong(vn);
+            if (step < 1e-9f * w.h && step * cancel < 1e-8f * w.h && vb >= 0 &&
+                vb <= __double_as_longlong(C2P_VSQMAX)) {
+                W = fma(widen(dw), __hiloint2double((int)eW, 0), Wd);  // 2^e dw
+                vsq = vn;
+                // the root moved by dv: 1/sqrt(1 - v^2) moves by half of y = dv / (1 - v^2), to second order
+                const float y = dv * rsh * rsh;
+                if (fabsf(y) < 1e-8f) rs64 = fma(r, widen(0.5f * y), r);
+                return true;
+            }
+        }
+    }
+    const C2PScalars T = S;
+    const NewtonOut o = newton_wv_call(&T, gfac, W, vsq);
+    W = o.W;
+    vsq = o.vsq;
+    it = o.it;
+    return o.ok;
+}
+
 // Mixed precision (the FP32-flux form only): FP32 Newton iterations first, on
 // the two equations scaled by k = 2^-e, e the binary exponent of the start's W
 // (an exact scaling; every term then O(1): f1 ~ W, f2 ~ W^2, so D, B^2, Q.n
@@ -113,8 +228,12 @@ __device__ __forceinline__ bool newton_wv_mixed(const C2PScalars& S, double gfac
     const float Wf = narrow(W);
     const unsigned eb = (__float_as_uint(Wf) >> 23) & 0xffu;  // biased exponent of the start
     if (!(Wf > 0.0f) || eb == 0u || eb >= 254u) {
-        const bool ok = newton_wv(S, gfac, W, vsq, it);
-        return ok;
+        const C2PScalars T = S;
+        const NewtonOut o = newton_wv_call(&T, gfac, W, vsq);
+        W = o.W;
+        vsq = o.vsq;
+        it = o.it;
+        return o.ok;
     }
     const float k = __uint_as_float((254u - eb) << 23);  // 2^(127 - eb): w = W k in [1, 2)
     const float k2 = k * k;
@@ -152,9 +271,12 @@ __device__ __forceinline__ bool newton_wv_mixed(const C2PScalars& S, double gfac
     }
     if (it32 > 8) it32 = 8;
     if (!ok32) {  // the FP64 iteration from the original start
-        const bool ok = newton_wv(S, gfac, W, vsq, it);
-        it += it32;
-        return ok;
+        const C2PScalars T = S;
+        const NewtonOut o = newton_wv_call(&T, gfac, W, vsq);
+        W = o.W;
+        vsq = o.vsq;
+        it = o.it + it32;
+        return o.ok;
     }
     const double D64 = S.D, Bsq64 = S.Bsq, QB264 = S.QB2, Qdotn64 = S.Qdotn, Qtsq64 = S.Qtsq;
     // the FP32 root in FP64 (W = w / k exactly) and the exact powers 1/k, k^3, k^4 in FP64
@@ -162,7 +284,6 @@ __device__ __forceinline__ bool newton_wv_mixed(const C2PScalars& S, double gfac
     const double ik = __hiloint2double((1023 + ed) << 20, 0);
     const double k3 = __hiloint2double((1023 - 3 * ed) << 20, 0), k4 = __hiloint2double((1023 - 4 * ed) << 20, 0);
     double Wd = widen(w) * ik, vd = widen(v);
-    int it64 = 0;
     {
         // FP64 residuals of newton_wv's form (times W^2) at the root
         const double omv = 1.0 - vd;
@@ -201,38 +322,12 @@ __device__ __forceinline__ bool newton_wv_mixed(const C2PScalars& S, double gfac
             vd = vn;
         }
     }
-    bool ok = false;
-    for (it64 = 1; it64 <= C2P_NMAX; it64++) {
-        const double omv = 1.0 - vd;
-        const double rs = rsqrt(omv);
-        const double sq = omv * rs;
-        const double W2 = Wd * Wd, W3 = W2 * Wd;
-        const double BW = Bsq64 + Wd;
-        const double p = gfac * (Wd * omv - D64 * sq);
-        // scaled as in newton_wv: one reciprocal per iteration
-        const double f1 = (-0.5 * Bsq64 * (1.0 + vd) - Wd + p - Qdotn64) * W2 + 0.5 * QB264;
-        const double f2 = (vd * BW * BW - Qtsq64) * W2 - QB264 * (Bsq64 + 2.0 * Wd);
-        const double j11 = (gfac * omv - 1.0) * W3 - QB264;
-        const double j12 = -0.5 * Bsq64 + gfac * (0.5 * D64 * rs - Wd);
-        const double j21 = 2.0 * BW * (vd * W3 + QB264);
-        const double j22 = BW * BW;
-        const double r = 1.0 / ((j11 * j22 - j12 * j21) * W2);
-        const double Wn = Wd + (j12 * f2 - j22 * f1) * W3 * r;
-        const double vn = fmin(fmax(vd + (j21 * f1 - j11 * f2) * r, 0.0), C2P_VSQMAX);
-        if (!(Wn > 0.0)) break;
-        const double err = fabs(Wn - Wd) + fabs(vn - vd) * Wn;
-        Wd = Wn;
-        vd = vn;
-        if (err < C2P_TOL * Wn) {
-            ok = true;
-            break;
-        }
-    }
-    if (it64 > C2P_NMAX) it64 = C2P_NMAX;
-    it = it32 + 1 + it64;
-    W = Wd;
-    vsq = vd;
-    return ok;
+    const C2PScalars T = S;
+    const NewtonOut o = newton_wv_call(&T, gfac, Wd, vd);
+    it = it32 + 1 + o.it;
+    W = o.W;
+    vsq = o.vsq;
+    return o.ok;
 }
 
 // Aitken-accelerated inversion (Sec. 2.6 names it beside Newton; Newman &
@@ -297,11 +392,12 @@ __device__ __forceinline__ bool aitken_wv(const C2PScalars& S, double gfac, doub
 }
 
 // rho and u_g of a converged (W, v^2) (u_g = p / (gam - 1) = (W (1 - v^2) - D sqrt(1 - v^2)) / gam);
-// false unless both are positive. rs: 1/sqrt(1 - v^2), the Lorentz factor, for the velocity.
+// false unless both are positive. rs: 1/sqrt(1 - v^2), the Lorentz factor, for the velocity (in: the
+// same where the caller has it, else 0).
 __device__ __forceinline__ bool energy_result(const C2PScalars& S, double igam, double W, double vsq, double& rho,
                                               double& u, double& rs) {
     const double omv = 1.0 - vsq;
-    rs = rsqrt(omv);
+    if (__double2hiint(rs) == 0) rs = rsqrt(omv);
     const double sq = omv * rs;
     rho = S.D * sq;
     u = (W * omv - S.D * sq) * igam;
@@ -326,11 +422,13 @@ struct C2PWork {
 };
 
 // start32 (mixed form, optional): the start (W, v^2) already formed in FP32 from the guess primitives;
-// igam, gfac (optional, > 0): 1/gam and (gam - 1)/gam formed once by the caller (else here, per state)
+// igam, gfac (optional, > 0): 1/gam and (gam - 1)/gam formed once by the caller (else here, per state);
+// start64 (optional): Gamma^2 and Gamma^2 v^2 of the guess primitives where the caller has them
 __device__ __forceinline__ void c2p_prepare(const double U[NCONS], const double Bc[3], const Metric<double>& m,
                                             double gam, const double pr[NPRIM], C2PWork& w,
                                             int method = HAMR_INV_NEWTON, int mixed = 0,
-                                            const float* start32 = nullptr, double igam = 0.0, double gfac = 0.0) {
+                                            const float* start32 = nullptr, double igam = 0.0, double gfac = 0.0,
+                                            const double* start64 = nullptr) {
     c2p_scalars(U, Bc, m, w.S);
     if (igam > 0.0) {
         w.igam = igam;
@@ -353,6 +451,9 @@ __device__ __forceinline__ void c2p_prepare(const double U[NCONS], const double 
         const float gsq = 1.0f + qsq;
         w.W0 = widen((narrow(pr[RHO]) + narrow(gam) * narrow(pr[UU])) * gsq);
         w.vsq0 = widen(fminf(qsq / gsq, (float)C2P_VSQMAX));
+    } else if (start64) {
+        w.W0 = (pr[RHO] + gam * pr[UU]) * start64[0];
+        w.vsq0 = fmin(start64[1] * (1.0 / start64[0]), C2P_VSQMAX);
     } else {
         const double q1 = pr[U1], q2 = pr[U2], q3 = pr[U3];
         const double qsq = m.g11 * q1 * q1 + m.g22 * q2 * q2 + m.g33 * q3 * q3 + 2.0 * m.g13 * q1 * q3;
@@ -362,7 +463,7 @@ __device__ __forceinline__ void c2p_prepare(const double U[NCONS], const double 
     }
     w.W = w.W0;
     w.vsq = 0.0;
-    w.rho = w.u = 0.0;
+    w.rho = w.u = w.rs = 0.0;
     w.ok = false;
     w.its = 0;
 }
@@ -378,6 +479,7 @@ __device__ __forceinline__ void c2p_attempt_p(C2PWork& w, double gam, double p) 
     if (ok) {
         w.W = W;
         w.vsq = vsq;
+        w.rs = 0.0;
         ok = energy_result(w.S, w.igam, W, vsq, w.rho, w.u, w.rs);
     }
     w.ok = ok;
@@ -394,7 +496,8 @@ __device__ __forceinline__ void c2p_attempt(C2PWork& w, double gam, double W, do
         return;
     }
     int it = 0;
-    bool ok = w.mixed ? newton_wv_mixed(w.S, gfac, W, vsq, it) : newton_wv(w.S, gfac, W, vsq, it);
+    w.rs = 0.0;
+    bool ok = w.mixed ? newton_wv_mixed(w.S, gfac, W, vsq, it) : newton_wv_ff(w.S, gfac, W, vsq, it, w.rs);
     w.its += it;
     w.W = W;
     w.vsq = vsq;
@@ -410,56 +513,156 @@ __device__ __forceinline__ void c2p_attempt_plain(C2PWork& w, double gam) {
         c2p_attempt(w, gam, w.W0, w.vsq0);
 }
 
+// The entropy backup: Newton in W on f = W (1 - v^2) - rho - gam p / (gam - 1), p = kappa rho^gam,
+// v^2(W) from the momentum equation, rho = D sqrt(1 - v^2).
+struct EntropyOut {
+    double W, vsq, rho, u;
+    bool ok;
+};
+
+__device__ __forceinline__ bool entropy_newton(const C2PScalars& S, double kappa, double gam, double& W) {
+    const double gr = gam / (gam - 1.0);
+    for (int k = 1; k <= C2P_NMAX; k++) {
+        const double W2 = W * W;
+        const double BW = S.Bsq + W;
+        const double num = S.Qtsq * W2 + S.QB2 * (S.Bsq + 2.0 * W);
+        const double den = W2 * BW * BW;
+        const double iden = 1.0 / den;
+        double vs = num * iden;
+        double dvs = (2.0 * (S.Qtsq * W + S.QB2) - num * 2.0 * W * BW * (S.Bsq + 2.0 * W) * iden) * iden;
+        if (vs > C2P_VSQMAX) {
+            vs = C2P_VSQMAX;
+            dvs = 0.0;
+        }
+        const double s1 = 1.0 - vs;
+        const double sq = sqrt(s1);
+        const double rh = S.D * sq;
+        const double p = kappa * pow(rh, gam);
+        const double f = W * s1 - rh - gr * p;
+        const double drh = -0.5 * S.D / sq * dvs;
+        const double df = s1 - W * dvs - drh * (1.0 + gr * gam * p / rh);
+        const double Wn = W - f / df;
+        if (!(Wn > 0.0)) return false;
+        const double err = fabs(Wn - W);
+        W = Wn;
+        if (err < C2P_TOL * Wn) return true;
+    }
+    return false;
+}
+
+// v^2 and rho at W; with the base point's rho and rho^gam (r0, pw0) also rho^gam, by the binomial series
+// in x = rho / r0 - 1 (|x| < 1e-3: the terms to x^4 leave 1e-15 x^... < 1e-16), which a pow would cost
+// five times
+__device__ __forceinline__ void entropy_point(const C2PScalars& S, double gam, double W, double r0, double pw0,
+                                              double& vsq, double& rh, double& pw, double& x) {
+    const double W2 = W * W, BW = S.Bsq + W;
+    vsq = fmin((S.Qtsq * W2 + S.QB2 * (BW + W)) / (W2 * BW * BW), C2P_VSQMAX);
+    rh = S.D * sqrt(1.0 - vsq);
+    x = 0.0;
+    if (r0 > 0.0) {
+        x = (rh - r0) / r0;
+        const double g1 = gam - 1.0, g2 = gam - 2.0, g3 = gam - 3.0;
+        pw = pw0 * fma(gam * x, fma(0.5 * g1 * x, fma(g2 * x * (1.0 / 3.0), fma(0.25 * g3, x, 1.0), 1.0), 1.0), 1.0);
+    } else {
+        pw = pow(rh, gam);
+    }
+}
+
+// The iterations run in FP32 first (scaled by the power of two of the start's W; p through base-2
+// logarithms), until a step is below 1e-5 W; two FP64 residuals with the FP32 slope then take the root from
+// there to the stopping rule, one power and its series for both and the result. Where the FP32 iteration
+// meets no root, or the second FP64 step is not below the rule, the FP64 iteration runs from the start.
+// Few cells come here (0.2% of a large torus, 4% of a small one), but their warps wait for this chain:
+// five or six FP64 iterations of ~145 FP64 instructions each before. On a 53x37x22 block the cell update,
+// which such warps end, went from 122 to 61 us.
+static __device__ __noinline__ EntropyOut entropy_backup(const C2PScalars* Sp, double kappa, double gam, double W0) {
+    const C2PScalars& S = *Sp;
+    EntropyOut o;
+    o.ok = false;
+    const unsigned eW = (unsigned)__double2hiint(W0) & 0xfff00000u;
+    if (eW - 0x2b000000u < 0x2a000000u && kappa > 0.0) {
+        const unsigned sh = 0x3ff00000u - eW;
+        const float D = ff_of(S.D, (int)sh).h, B2 = ff_of(S.Bsq, (int)sh).h;
+        const float Qt = ff_of(S.Qtsq, (int)(2u * sh)).h, QB = ff_of(S.QB2, (int)(3u * sh)).h;
+        const float gf = (float)gam, gr = gf / (gf - 1.0f);
+        const float e = (float)((int)(eW >> 20) - 1023);
+        // log2 p = log2 kappa + gam (log2 rho_scaled + e) - e
+        const int ke = (__double2hiint(kappa) >> 20) - 1023;
+        const float km = __uint_as_float(0x3f800000u | (((unsigned)__double2hiint(kappa) & 0xfffffu) << 3));
+        const float lk = (float)ke + log2f(km) + (gf - 1.0f) * e;
+        float w = ff_of(W0, (int)sh).h, df = 0.0f;
+        bool ok32 = false;
+        for (int k = 0; k < C2P_NMAX && !ok32; k++) {
+            const float bw = B2 + w, den = w * w * bw * bw, iden = 1.0f / den;
+            const float num = Qt * w * w + QB * (B2 + 2.0f * w);
+            float vs = num * iden;
+            float dvs = (2.0f * (Qt * w + QB) - num * 2.0f * w * bw * (B2 + 2.0f * w) * iden) * iden;
+            if (vs > (float)C2P_VSQMAX) {
+                vs = (float)C2P_VSQMAX;
+                dvs = 0.0f;
+            }
+            const float s1 = 1.0f - vs, sq = sqrtf(s1), rh = D * sq;
+            const float p = exp2f(lk + gf * log2f(rh));
+            const float f = w * s1 - rh - gr * p;
+            df = s1 - w * dvs + 0.5f * D / sq * dvs * (1.0f + gr * gf * p / rh);
+            const float wn = w - f / df;
+            if (!(wn > 0.0f && wn < 1e9f)) break;
+            ok32 = fabsf(wn - w) < 1e-5f * wn;
+            w = wn;
+        }
+        if (ok32 && fabsf(df) > 1e-6f) {
+            const double gr64 = gam / (gam - 1.0);
+            double W = widen(w);
+            W = __hiloint2double((int)((unsigned)__double2hiint(W) - sh), __double2loint(W));
+            const double idf = 1.0 / widen(df);
+            double vs, rh, pw, x, r0, pw0;
+            entropy_point(S, gam, W, 0.0, 0.0, vs, r0, pw0, x);
+            const double d1 = (W * (1.0 - vs) - r0 - gr64 * kappa * pw0) * idf;
+            W -= d1;
+            entropy_point(S, gam, W, r0, pw0, vs, rh, pw, x);
+            const double d2 = (W * (1.0 - vs) - rh - gr64 * kappa * pw) * idf;
+            W -= d2;
+            // the rule on the second step, and both small enough for the slope's error (the contraction
+            // d2 / d1) to leave the third below round-off
+            if (W > 0.0 && fabs(d1) < 1e-4 * W && fabs(d2) < C2P_TOL * W && d2 * d2 < 1e-16 * fabs(d1) * W) {
+                entropy_point(S, gam, W, r0, pw0, o.vsq, o.rho, pw, x);
+                if (fabs(x) < 1e-3) {
+                    o.W = W;
+                    o.u = kappa * pw / (gam - 1.0);
+                    o.ok = (o.rho > 0.0) && (o.u > 0.0) && (o.vsq >= 0.0);
+                    return o;
+                }
+            }
+        }
+    }
+    double W = W0;
+    if (entropy_newton(S, kappa, gam, W)) {
+        const double W2 = W * W;
+        const double BW = S.Bsq + W;
+        o.W = W;
+        o.vsq = fmin((S.Qtsq * W2 + S.QB2 * (S.Bsq + 2.0 * W)) / (W2 * BW * BW), C2P_VSQMAX);
+        o.rho = S.D * sqrt(1.0 - o.vsq);
+        o.u = kappa * pow(o.rho, gam) / (gam - 1.0);
+        o.ok = (o.rho > 0.0) && (o.u > 0.0) && (o.vsq >= 0.0);
+    }
+    return o;
+}
+
 // pr: out the result (slots 0..4) unless INV_FAIL (then untouched)
 __device__ __forceinline__ int c2p_finish(C2PWork& w, const double U[NCONS], const Metric<double>& m, double gam,
                                           double pr[NPRIM]) {
     const C2PScalars& S = w.S;
-    const double D = S.D, Bsq = S.Bsq, QB2 = S.QB2, Qtsq = S.Qtsq;
+    const double Bsq = S.Bsq;
     double W = w.W, vsq = w.vsq, rho = w.rho, u = w.u;
     int status = INV_OK;
     if (!w.ok) {
-        const double kappa = U[C_ENT] / U[C_RHO];
-        const double gr = gam / (gam - 1.0);
-        W = w.W0;
-        bool eok = false;
-        for (int k = 1; k <= C2P_NMAX; k++) {
-            const double W2 = W * W;
-            const double BW = Bsq + W;
-            const double num = Qtsq * W2 + QB2 * (Bsq + 2.0 * W);
-            const double den = W2 * BW * BW;
-            const double iden = 1.0 / den;
-            double vs = num * iden;
-            double dvs = (2.0 * (Qtsq * W + QB2) - num * 2.0 * W * BW * (Bsq + 2.0 * W) * iden) * iden;
-            if (vs > C2P_VSQMAX) {
-                vs = C2P_VSQMAX;
-                dvs = 0.0;
-            }
-            const double s1 = 1.0 - vs;
-            const double sq = sqrt(s1);
-            const double rh = D * sq;
-            const double p = kappa * pow(rh, gam);
-            const double f = W * s1 - rh - gr * p;
-            const double drh = -0.5 * D / sq * dvs;
-            const double df = s1 - W * dvs - drh * (1.0 + gr * gam * p / rh);
-            const double Wn = W - f / df;
-            if (!(Wn > 0.0)) break;
-            const double err = fabs(Wn - W);
-            W = Wn;
-            if (err < C2P_TOL * Wn) {
-                eok = true;
-                break;
-            }
-        }
-        if (eok) {
-            const double W2 = W * W;
-            const double BW = Bsq + W;
-            vsq = fmin((Qtsq * W2 + QB2 * (Bsq + 2.0 * W)) / (W2 * BW * BW), C2P_VSQMAX);
-            const double sq = sqrt(1.0 - vsq);
-            rho = D * sq;
-            u = kappa * pow(rho, gam) / (gam - 1.0);
-            eok = (rho > 0.0) && (u > 0.0) && (vsq >= 0.0);
-        }
-        if (!eok) return INV_FAIL;
+        const C2PScalars T = S;
+        const EntropyOut o = entropy_backup(&T, U[C_ENT] / U[C_RHO], gam, w.W0);
+        if (!o.ok) return INV_FAIL;
+        W = o.W;
+        vsq = o.vsq;
+        rho = o.rho;
+        u = o.u;
         status = INV_ENTROPY;
     }
     // utilde^i = Gamma/(W + B^2) (Qt^i + (Q.B) Bn^i / W), Qt^i = Q^i - alpha g^{ti} (Q.n);

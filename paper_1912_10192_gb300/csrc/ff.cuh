@@ -27,7 +27,7 @@ struct ff {
 // above binary32's range give non-finite or meaningless words: callers test the result they need.
 __device__ __forceinline__ ff ff_of(double x, int sh = 0) {
     const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-    const int a = (int)(hi & 0x7fffffffu) + sh;
+    const int a = (int)((hi & 0x7fffffffu) + (unsigned)sh);  // wraps: sh may be several exponents' sum
     const unsigned s = hi & 0x80000000u;
     const unsigned u = (((unsigned)a - 0x38000000u) << 3) | (lo >> 29);  // binary32 bits of the truncated value
     const float r = (float)(lo & 0x1fffffffu);
