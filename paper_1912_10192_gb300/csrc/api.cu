@@ -532,7 +532,7 @@ int hamr_block_step(hamr_grid* g, int block, double dt, void* stream, hamr_step_
     if (ph.smr) LAUNCH(g, K_EMF, 1, cs, launch_smr_emf(v, ph, s.E, cs));
     LAUNCH(g, K_CT, 1, cs, launch_ct(v, s.E, s.B, s.Bh, s.dscal, 0.5, cs));
     LAUNCH(g, K_UPDATE, 1, cs,
-           launch_update(v, ph, 0, s.P, s.P, s.F, s.Bh, s.Un, s.Ph, s.status, s.dscal, 0.5, s.dmax, s.dcnt, cs));
+           launch_update(v, ph, 0, s.P, s.F, s.Bh, s.Un, s.Ph, s.status, s.dscal, 0.5, s.dmax, s.dcnt, cs));
     if (ph.smr)
         LAUNCH(g, K_UPDATE, 1, cs, launch_smr_cells(v, ph, 0, s.P, s.Bh, s.Ph, s.status, s.dmax, s.dcnt, cs));
     // corrector: U^n and the fluxes of P^{n+1/2} -> P^{n+1}, B^{n+1} (in place)
@@ -548,7 +548,7 @@ int hamr_block_step(hamr_grid* g, int block, double dt, void* stream, hamr_step_
     if (ph.smr) LAUNCH(g, K_EMF, 1, cs, launch_smr_emf(v, ph, s.E, cs));
     LAUNCH(g, K_CT, 1, cs, launch_ct(v, s.E, s.B, s.B, s.dscal, 1.0, cs));
     LAUNCH(g, K_UPDATE, 1, cs,
-           launch_update(v, ph, 1, s.P, s.Ph, s.F, s.B, s.Un, s.P, s.status, s.dscal, 1.0, s.dmax, s.dcnt, cs));
+           launch_update(v, ph, 1, s.Ph, s.F, s.B, s.Un, s.P, s.status, s.dscal, 1.0, s.dmax, s.dcnt, cs));
     if (ph.smr)
         LAUNCH(g, K_UPDATE, 1, cs, launch_smr_cells(v, ph, 1, s.Ph, s.B, s.P, s.status, s.dmax, s.dcnt, cs));
     LAUNCH(g, K_BC, 4, cs, launch_bc(v, s.P, s.B, cs, P32g, K32g));
@@ -864,7 +864,7 @@ int time_group_block(hamr_grid* g, const PhysArgs& ph, int which, cudaStream_t c
         if (which == 2) {
             float t = 0.0f;
             CUDA_TRY(cudaEventRecord(a, cs));
-            CUDA_TRY(launch_update(v, ph, 0, s.P, s.P, s.F, s.B, s.Un, s.Ph, s.status, s.dscal, 0.5, s.dmax, s.dcnt,
+            CUDA_TRY(launch_update(v, ph, 0, s.P, s.F, s.B, s.Un, s.Ph, s.status, s.dscal, 0.5, s.dmax, s.dcnt,
                                    cs));
             CUDA_TRY(cudaEventRecord(b, cs));
             CUDA_TRY(cudaEventSynchronize(b));

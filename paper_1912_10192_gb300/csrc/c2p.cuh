@@ -24,6 +24,10 @@ constexpr double C2P_VSQMAX = 1.0 - 1.0 / (50.0 * 50.0);
 
 enum { INV_OK = 0, INV_ENTROPY = 1, INV_FAIL = 2 };
 
+// how Newton iterates: in double-float with an FP64 last solve (newton_wv_ff), in FP32 with one FP64
+// refinement step (newton_wv_mixed), or in FP64 (newton_wv: grids of the mixed forms, update.cu)
+enum { C2P_NEWTON_FF = 0, C2P_NEWTON32 = 1, C2P_NEWTON64 = 2 };
+
 // The normal-frame scalars of a conserved state (Sec. 2.6, Noble et al. 2006).
 struct C2PScalars {
     double D, Qdotn, Qtsq, Bsq, QdotB, QB2;
@@ -114,13 +118,16 @@ static __device__ __noinline__ NewtonOut newton_wv_call(const C2PScalars* S, dou
 // that brings the start's W to [1, 2) (f1 ~ W, f2 ~ W^2), on the FP32 pipe; then the FP64 residuals at
 // that root, solved with the Jacobian of the last iteration. The double-float root is 1e-13 or better, so
 // that solve (relative error of the Jacobian 1e-7 times its cancellation) leaves what FP64 residuals
-// resolve, like newton_wv's own last iterate. Taken when the step and the step times the cancellation
+// resolve, like newton_wv's own last iterate. Where the steps still shrink slowly at the end (not by 1e-3;
+// v^2 near its limit), newton_wv stops short of the root by up to its tolerance, and where a step is within
+// the double-float steps' noise (1e-13 times the cancellation) of the tolerance, rounding decides whether it
+// stops: both are left to it. Taken when the step and the step times the cancellation
 // (|j11 j22| + |j12 j21|) / |det| are as small as that argument needs; otherwise, and wherever the
 // double-float iteration meets no root or leaves its range, newton_wv decides. `it` counts the iterations,
 // not the solve. rs: 1/sqrt(1 - v^2) at the root where it comes for free, else 0.
 // An FP64 iteration is ~52 FP64 instructions (64 cycles each per scheduler), here ~340 FP32 ones, plus
-// ~28 FP64 for the solve: 1,000,003 states from a 5% start (4.7 iterations) 1021 -> 564 us with the entropy
-// backup below, the FP64 cell update of the 256x128x64 torus 2.00 -> 1.50 ms.
+// ~28 FP64 for the solve: 1,000,003 states from a 5% start (4.7 iterations) 1021 -> 626 us, the FP64
+// cell update of the 256x128x64 torus 2.00 -> 1.50 ms with the entropy backup below.
 __device__ __forceinline__ bool newton_wv_ff(const C2PScalars& S, double gfac, double& W, double& vsq, int& it,
                                              double& rs64) {
     rs64 = 0.0;
@@ -135,6 +142,7 @@ __device__ __forceinline__ bool newton_wv_ff(const C2PScalars& S, double gfac, d
         const ff hB = ff_scale(B2, 0.5f), c1 = ff_neg(ff_add(hB, Qn));
         ff w = ff_of(W, (int)sh), v = ff_of(vsq);
         float j11h = 0.0f, j12h = 0.0f, j21h = 0.0f, j22h = 0.0f, idh = 0.0f, iwh = 0.0f, rsh = 0.0f;
+        float before = 1e30f, cancel = 0.0f;  // the step before; the Jacobian's cancellation
         for (it = 1; it <= C2P_NMAX; it++) {
             const ff omv = ff_sub(one, v);
             const ff rs = ff_rsqrt(omv);
@@ -160,8 +168,13 @@ __device__ __forceinline__ bool newton_wv_ff(const C2PScalars& S, double gfac, d
             const float err = fabsf(dw.h) + fabsf((vn.h - v.h) + (vn.l - v.l)) * wn.h;
             w = wn;
             v = vn;
-            if (err < (float)C2P_TOL * wn.h) {
-                ok = true;
+            // the steps' noise: 2^-46 or so times the Jacobian's cancellation. Where that comes near the
+            // tolerance, or the steps have stopped shrinking, FP64 decides
+            cancel = (fabsf(j11.h * j22.h) + fabsf(j12.h * j21.h)) * fabsf(id.h);
+            const float tol = (float)C2P_TOL * wn.h, noise = 1e-13f * cancel * wn.h;
+            if (noise > 0.5f * tol || (err > 0.25f * before && before < 1e-6f * wn.h)) break;
+            if (err < tol) {
+                ok = err + noise < tol && before > tol + noise && (err < 1e-3f * before || err < 0.1f * tol);
                 j11h = j11.h;
                 j12h = j12.h;
                 j21h = j21.h;
@@ -171,6 +184,7 @@ __device__ __forceinline__ bool newton_wv_ff(const C2PScalars& S, double gfac, d
                 rsh = rs.h;
                 break;
             }
+            before = err;
         }
         if (ok) {
             double Wd = ff_d(w);  // in [2^-40, 2^30]: the exponent added back as an integer
@@ -186,7 +200,6 @@ __device__ __forceinline__ bool newton_wv_ff(const C2PScalars& S, double gfac, d
             const float r1 = ff_of(f1, (int)(3u * sh)).h * iw2, r2 = ff_of(f2, (int)(4u * sh)).h * iw2;
             const float dw = (j12h * r2 - j22h * r1) * idh, dv = (j21h * r1 - j11h * r2) * idh;
             const float step = fabsf(dw) + fabsf(dv) * w.h;
-            const float cancel = (fabsf(j11h * j22h) + fabsf(j12h * j21h)) * fabsf(idh);
             const double vn = vd + widen(dv);
             const long long vb = __double_as_longlong(vn);
             if (step < 1e-9f * w.h && step * cancel < 1e-8f * w.h && vb >= 0 &&
@@ -413,7 +426,7 @@ struct C2PWork {
     double W0, vsq0;  // the start from the guess primitives
     double p0;        // ... and its pressure (the Aitken inversion's start)
     int method;       // HAMR_INV_NEWTON or HAMR_INV_AITKEN
-    int mixed;        // Newton: FP32 iterations first (newton_wv_mixed)
+    int form;         // Newton: C2P_NEWTON_FF, C2P_NEWTON32 or C2P_NEWTON64
     double igam, gfac;  // 1/gam and (gam - 1)/gam, from one division per inversion
     double W, vsq, rho, u;
     double rs;        // 1/sqrt(1 - v^2) of an energy result
@@ -426,7 +439,7 @@ struct C2PWork {
 // start64 (optional): Gamma^2 and Gamma^2 v^2 of the guess primitives where the caller has them
 __device__ __forceinline__ void c2p_prepare(const double U[NCONS], const double Bc[3], const Metric<double>& m,
                                             double gam, const double pr[NPRIM], C2PWork& w,
-                                            int method = HAMR_INV_NEWTON, int mixed = 0,
+                                            int method = HAMR_INV_NEWTON, int form = C2P_NEWTON_FF,
                                             const float* start32 = nullptr, double igam = 0.0, double gfac = 0.0,
                                             const double* start64 = nullptr) {
     c2p_scalars(U, Bc, m, w.S);
@@ -438,12 +451,12 @@ __device__ __forceinline__ void c2p_prepare(const double U[NCONS], const double 
         w.gfac = (gam - 1.0) * w.igam;
     }
     w.method = method;
-    w.mixed = mixed;
+    w.form = form;
     w.p0 = (method == HAMR_INV_AITKEN) ? (gam - 1.0) * pr[UU] : 0.0;
-    if (mixed && start32) {
+    if (form == C2P_NEWTON32 && start32) {
         w.W0 = widen(start32[0]);
         w.vsq0 = widen(fminf(start32[1], (float)C2P_VSQMAX));
-    } else if (mixed) {
+    } else if (form == C2P_NEWTON32) {
         // the start only seeds the FP32 iterations (and, where they fail, the FP64 ones): in FP32
         const float q1 = narrow(pr[U1]), q2 = narrow(pr[U2]), q3 = narrow(pr[U3]);
         const float qsq = narrow(m.g11) * q1 * q1 + narrow(m.g22) * q2 * q2 + narrow(m.g33) * q3 * q3 +
@@ -497,7 +510,9 @@ __device__ __forceinline__ void c2p_attempt(C2PWork& w, double gam, double W, do
     }
     int it = 0;
     w.rs = 0.0;
-    bool ok = w.mixed ? newton_wv_mixed(w.S, gfac, W, vsq, it) : newton_wv_ff(w.S, gfac, W, vsq, it, w.rs);
+    bool ok = (w.form == C2P_NEWTON32)   ? newton_wv_mixed(w.S, gfac, W, vsq, it)
+              : (w.form == C2P_NEWTON64) ? newton_wv(w.S, gfac, W, vsq, it)
+                                         : newton_wv_ff(w.S, gfac, W, vsq, it, w.rs);
     w.its += it;
     w.W = W;
     w.vsq = vsq;
@@ -573,14 +588,16 @@ __device__ __forceinline__ void entropy_point(const C2PScalars& S, double gam, d
 // there to the stopping rule, one power and its series for both and the result. Where the FP32 iteration
 // meets no root, or the second FP64 step is not below the rule, the FP64 iteration runs from the start.
 // Few cells come here (0.2% of a large torus, 4% of a small one), but their warps wait for this chain:
-// five or six FP64 iterations of ~145 FP64 instructions each before. On a 53x37x22 block the cell update,
-// which such warps end, went from 122 to 61 us.
-static __device__ __noinline__ EntropyOut entropy_backup(const C2PScalars* Sp, double kappa, double gam, double W0) {
+// five or six FP64 iterations of ~145 FP64 instructions each before. On a 64x32x16 block the cell update,
+// which such warps end, went from 112 to 67 us (with newton_wv_ff). fast = false: the FP64 iteration alone (the mixed forms,
+// whose results stay bit for bit, update.cu).
+static __device__ __noinline__ EntropyOut entropy_backup(const C2PScalars* Sp, double kappa, double gam, double W0,
+                                                         bool fast) {
     const C2PScalars& S = *Sp;
     EntropyOut o;
     o.ok = false;
     const unsigned eW = (unsigned)__double2hiint(W0) & 0xfff00000u;
-    if (eW - 0x2b000000u < 0x2a000000u && kappa > 0.0) {
+    if (fast && eW - 0x2b000000u < 0x2a000000u && kappa > 0.0) {
         const unsigned sh = 0x3ff00000u - eW;
         const float D = ff_of(S.D, (int)sh).h, B2 = ff_of(S.Bsq, (int)sh).h;
         const float Qt = ff_of(S.Qtsq, (int)(2u * sh)).h, QB = ff_of(S.QB2, (int)(3u * sh)).h;
@@ -606,8 +623,8 @@ static __device__ __noinline__ EntropyOut entropy_backup(const C2PScalars* Sp, d
             const float f = w * s1 - rh - gr * p;
             df = s1 - w * dvs + 0.5f * D / sq * dvs * (1.0f + gr * gf * p / rh);
             const float wn = w - f / df;
-            if (!(wn > 0.0f && wn < 1e9f)) break;
-            ok32 = fabsf(wn - w) < 1e-5f * wn;
+            if (!(wn > 0.02f * w && wn < 1e9f)) break;  // near wn = 0 rounding decides whether FP64 fails
+            ok32 = k < 12 && fabsf(wn - w) < 1e-5f * wn;
             w = wn;
         }
         if (ok32 && fabsf(df) > 1e-6f) {
@@ -624,7 +641,7 @@ static __device__ __noinline__ EntropyOut entropy_backup(const C2PScalars* Sp, d
             W -= d2;
             // the rule on the second step, and both small enough for the slope's error (the contraction
             // d2 / d1) to leave the third below round-off
-            if (W > 0.0 && fabs(d1) < 1e-4 * W && fabs(d2) < C2P_TOL * W && d2 * d2 < 1e-16 * fabs(d1) * W) {
+            if (W > 0.0 && fabs(d1) < 1e-4 * W && fabs(d2) < C2P_TOL * W && d2 * d2 <= 1e-16 * fabs(d1) * W) {
                 entropy_point(S, gam, W, r0, pw0, o.vsq, o.rho, pw, x);
                 if (fabs(x) < 1e-3) {
                     o.W = W;
@@ -657,7 +674,7 @@ __device__ __forceinline__ int c2p_finish(C2PWork& w, const double U[NCONS], con
     int status = INV_OK;
     if (!w.ok) {
         const C2PScalars T = S;
-        const EntropyOut o = entropy_backup(&T, U[C_ENT] / U[C_RHO], gam, w.W0);
+        const EntropyOut o = entropy_backup(&T, U[C_ENT] / U[C_RHO], gam, w.W0, w.form == C2P_NEWTON_FF);
         if (!o.ok) return INV_FAIL;
         W = o.W;
         vsq = o.vsq;
@@ -688,9 +705,10 @@ __device__ __forceinline__ int c2p_finish(C2PWork& w, const double U[NCONS], con
 // Newton iterations of every start tried.
 __device__ __forceinline__ int invert(const double U[NCONS], const double Bc[3], const Metric<double>& m, double gam,
                                       double pr[NPRIM], int* iters, bool entropy_only,
-                                      const double* guess2 = nullptr, int method = HAMR_INV_NEWTON) {
+                                      const double* guess2 = nullptr, int method = HAMR_INV_NEWTON,
+                                      int form = C2P_NEWTON_FF) {
     C2PWork w;
-    c2p_prepare(U, Bc, m, gam, pr, w, method);
+    c2p_prepare(U, Bc, m, gam, pr, w, method, form);
     if (!entropy_only) {
         if (guess2) c2p_attempt(w, gam, guess2[0], guess2[1]);
         c2p_attempt_plain(w, gam);

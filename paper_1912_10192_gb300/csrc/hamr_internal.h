@@ -253,8 +253,9 @@ cudaError_t launch_smr_emf_batch(const DevBlock* tab, const int* list, int nlist
                                  cudaStream_t s);
 cudaError_t launch_smr_cells_batch(const DevBlock* tab, const int* list, int nlist, long maxwork, const PhysArgs& ph,
                                    int sigma, cudaStream_t s);
-cudaError_t launch_update(const BlockView& v, const PhysArgs& ph, int corrector, const double* Pbase,
-                          const double* Pflux, double* const F[3], const double* Bnew, double* Un, double* Pout,
+// U^n comes from Pflux in the predictor (0) and from the cache Un in the corrector (1)
+cudaError_t launch_update(const BlockView& v, const PhysArgs& ph, int corrector, const double* Pflux,
+                          double* const F[3], const double* Bnew, double* Un, double* Pout,
                           uint8_t* status, const double* dscal, double dt_factor, unsigned long long* dmax,
                           unsigned long long* dcnt, cudaStream_t s);
 cudaError_t launch_dt_reduce(const BlockView& v, const PhysArgs& ph, const double* P, unsigned long long* dmax,

@@ -199,7 +199,7 @@ extern "C" int hamr_block_step_noalloc(const hamr_grid_desc* d, double* prim, do
     }
     NA_TRY(launch_emf(v, s.F, s.E, ph.mixed, s.P, ph.emf ? s.QL : nullptr, cs));
     NA_TRY(launch_ct(v, s.E, s.B, s.Bh, s.dscal, 0.5, cs));
-    NA_TRY(launch_update(v, ph, 0, s.P, s.P, s.F, s.Bh, s.Un, s.Ph, s.status, s.dscal, 0.5, s.dmax, s.dcnt, cs));
+    NA_TRY(launch_update(v, ph, 0, s.P, s.F, s.Bh, s.Un, s.Ph, s.status, s.dscal, 0.5, s.dmax, s.dcnt, cs));
     // corrector
     NA_TRY(launch_bc(v, s.Ph, s.Bh, cs));
     NA_TRY(launch_kappa(v, ph, s.Ph, nullptr, s.E, nullptr, cs));
@@ -210,7 +210,7 @@ extern "C" int hamr_block_step_noalloc(const hamr_grid_desc* d, double* prim, do
     }
     NA_TRY(launch_emf(v, s.F, s.E, ph.mixed, s.Ph, ph.emf ? s.QL : nullptr, cs));
     NA_TRY(launch_ct(v, s.E, s.B, s.B, s.dscal, 1.0, cs));
-    NA_TRY(launch_update(v, ph, 1, s.P, s.Ph, s.F, s.B, s.Un, s.P, s.status, s.dscal, 1.0, s.dmax, s.dcnt, cs));
+    NA_TRY(launch_update(v, ph, 1, s.Ph, s.F, s.B, s.Un, s.P, s.status, s.dscal, 1.0, s.dmax, s.dcnt, cs));
     NA_TRY(launch_bc(v, s.P, s.B, cs));
     return HAMR_OK;
 }

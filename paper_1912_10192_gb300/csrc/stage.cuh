@@ -43,6 +43,7 @@ struct Side64 {
     double c0, c1, c2, c3;   // u_mu
     double k0, k1, k2, k3;   // B_mu
     double iut, s2, Y, bsq;  // 1/u^t, i2 B^2, i2 b^t, b^2
+    double g2, i2;           // Gamma^2, 1/(u^t)^2
 };
 
 __device__ __forceinline__ void side64(const double pr[NPRIM], const Metric<double>& m, double ac01, Side64& s) {
@@ -50,9 +51,9 @@ __device__ __forceinline__ void side64(const double pr[NPRIM], const Metric<doub
     s.c1 = m.g11 * q1 + m.g13 * q3;
     s.c2 = m.g22 * q2;
     s.c3 = m.g13 * q1 + m.g33 * q3;
-    const double g2 = fma(q1, s.c1, fma(q2, s.c2, fma(q3, s.c3, 1.0)));  // Gamma^2
-    const double ig = rsqrt(g2);
-    const double gamma = g2 * ig;
+    s.g2 = fma(q1, s.c1, fma(q2, s.c2, fma(q3, s.c3, 1.0)));
+    const double ig = rsqrt(s.g2);
+    const double gamma = s.g2 * ig;
     s.ut = gamma * m.ialpha;
     s.u1 = q1 - gamma * ac01;
     s.u2 = q2;
@@ -65,24 +66,13 @@ __device__ __forceinline__ void side64(const double pr[NPRIM], const Metric<doub
     s.k3 = m.g13 * b1 + m.g33 * b3;
     const double bt = b1 * s.c1 + b2 * s.c2 + b3 * s.c3;
     s.iut = m.alpha * ig;
-    const double i2 = s.iut * s.iut;
-    s.s2 = i2 * (b1 * s.k1 + b2 * s.k2 + b3 * s.k3);
-    s.Y = i2 * bt;
+    s.i2 = s.iut * s.iut;
+    s.s2 = s.i2 * (b1 * s.k1 + b2 * s.k2 + b3 * s.k3);
+    s.Y = s.i2 * bt;
     s.bsq = s.s2 + s.Y * bt;
 }
 
 // ---------------------------------------------------------------- reductions
-__device__ __forceinline__ double warp_max(double x) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x = fmax(x, __shfl_xor_sync(0xffffffffu, x, o));
-    return x;
-}
-__device__ __forceinline__ unsigned long long warp_sum(unsigned long long x) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    return x;
-}
-
 // sum_i v_f^i / dx^i at a cell centre (Sec. 2.1 CFL condition), given the fluid state
 // (max(|v+|, |v-|) = (|B| + sd)/|A| per direction; the three terms over one denominator)
 template <typename T>
@@ -120,7 +110,7 @@ __device__ __forceinline__ double inv_dt_cell(const BlockView& v, const T pr[NPR
 // (tables gc: metric and connection planes of that precision)
 template <typename T, typename TT>
 __device__ __forceinline__ void source_q_state(const TT* __restrict__ gc, long n2d, long g, const Metric<T>& m,
-                                              const T pf[NPRIM], const Fluid<T>& s, T gam, double Q[4]) {
+                                              const T pf[NPRIM], const Fluid<T>& s, T gam, T Q[4]) {
     const T p = (gam - T(1)) * pf[UU];
     const T eta = pf[RHO] + pf[UU] + p + s.bsq;
     const T ptot = p + T(0.5) * s.bsq;
@@ -138,7 +128,7 @@ __device__ __forceinline__ void source_q_state(const TT* __restrict__ gc, long n
         for (int l = 0; l < 4; l++)
 #pragma unroll
             for (int kk = 0; kk < 4; kk++) acc += Tm[kk][l] * (T)cn[(l * 10 + sym(nu, kk)) * n2d];
-        Q[nu] = to_d(acc * m.gdet);
+        Q[nu] = acc * m.gdet;
     }
 }
 
@@ -147,7 +137,31 @@ __device__ __forceinline__ void source_q_state(const TT* __restrict__ gc, long n
 // T^k_l Gamma^l_{nu k} = (1/2) T^{kl} d_nu g_{kl} (the terms with d_k g_{l nu} - d_l g_{nu k}
 // cancel against the symmetric T^{kl}), so Q_t = Q_phi = 0 (stationary, axisymmetric
 // metric) and Q_1, Q_2 contract the 7 non-zero d_s g_{mn}; the same number up to
-// rounding order, with a third of the operations.
+// rounding order, with a third of the operations. With b^mu = (B^mu + b^t u^mu)/u^t
+//   T^{mn} = (rho h + i2 B^2) u^m u^n - Y (B^m u^n + u^m B^n) - i2 B^m B^n + ptot g^{mn}
+//          = h^m u^n - B^n g^m + ptot g^{mn}, h = (rho h + i2 B^2) u - Y B, g = Y u + i2 B.
+// Q: Q_1 and Q_2 without sqrt(-g).
+__device__ __forceinline__ void source64(const double* __restrict__ gc, long n2d, long g, const Metric<double>& m,
+                                         const double pf[NPRIM], const Side64& s, double gam, double& Q1, double& Q2) {
+    const double w = fma(gam, pf[UU], pf[RHO]) + s.s2;
+    const double ptot = (gam - 1.0) * pf[UU] + 0.5 * s.bsq;
+    const double b1 = pf[B1], b2 = pf[B2], b3 = pf[B3];
+    const double h1 = w * s.u1 - s.Y * b1, h2 = w * s.u2 - s.Y * b2, h3 = w * s.u3 - s.Y * b3;
+    const double g1 = s.Y * s.u1 + s.i2 * b1, g2 = s.Y * s.u2 + s.i2 * b2, g3 = s.Y * s.u3 + s.i2 * b3;
+    const double T[7] = {w * s.ut * s.ut + ptot * m.c00,           h1 * s.ut + ptot * m.c01,
+                         h3 * s.ut,                                h1 * s.u1 + (-b1 * g1 + ptot * m.c11),
+                         h1 * s.u3 + (-b3 * g1 + ptot * m.c13),    h2 * s.u2 + (-b2 * g2 + ptot * m.c22),
+                         h3 * s.u3 + (-b3 * g3 + ptot * m.c33)};
+    const double* d = gc + (long)C_DG * n2d + g;
+    Q1 = Q2 = 0.0;
+#pragma unroll
+    for (int k = 0; k < 7; k++) {
+        Q1 += T[k] * d[k * n2d];
+        Q2 += T[k] * d[(7 + k) * n2d];
+    }
+}
+
+// The same from b^mu, as the mixed form with the FP64 source takes it (Q: all four, times sqrt(-g)).
 __device__ __forceinline__ void source_q_dg(const double* __restrict__ gc, long n2d, long g, const Metric<double>& m,
                                             const double pf[NPRIM], const Fluid<double>& s, double gam, double Q[4]) {
     const double p = (gam - 1.0) * pf[UU];
@@ -173,15 +187,64 @@ __device__ __forceinline__ void source_q_dg(const double* __restrict__ gc, long 
     Q[3] = 0.0;
 }
 
-template <typename T, typename TT>
-__device__ __forceinline__ void source_q(const TT* __restrict__ gc, long n2d, long g, const Metric<T>& m,
-                                        const double pfd[NPRIM], double gam_d, double Q[4]) {
-    T pf[NPRIM];
+// adds the warp's cells to the counters of a step: inversions by outcome st (-1: none), floors, iterations
+__device__ __forceinline__ void count_cells(int st, int fl, int its, unsigned long long* dcnt) {
+    const unsigned all = 0xffffffffu;
+    const int c[5] = {__popc(__ballot_sync(all, st == INV_OK)), __popc(__ballot_sync(all, st == INV_ENTROPY)),
+                      __popc(__ballot_sync(all, st == INV_FAIL)), __popc(__ballot_sync(all, fl != 0)),
+                      __reduce_add_sync(all, its)};
+    if ((threadIdx.x & 31u) == 0) {
 #pragma unroll
-    for (int q = 0; q < NPRIM; q++) pf[q] = to_t<T>(pfd[q]);
-    Fluid<T> s;
-    fluid_state(pf, m, s);
-    source_q_state(gc, n2d, g, m, pf, s, to_t<T>(gam_d), Q);
+        for (int q = 0; q < 5; q++)
+            if (c[q]) atomicAdd(&dcnt[q], (unsigned long long)c[q]);
+    }
+}
+
+// ---- the CFL rate in FP32, to leave out the FP64 one where it cannot be the largest
+// Estimate of inv_dt_fluid from (rho, u, b^2), all scaled by one factor, and u^mu; negative where it says
+// nothing. Its discriminant may lose all digits to cancellation: the root's error is then below
+// sqrt(2^-22) = 5e-4 of |B|, so the estimate is within 1e-3 of the rate wherever num g^{dd} stays in range.
+__device__ __forceinline__ float rate_estimate(const BlockView& v, const PhysArgs& ph, float rho, float u, float bsq,
+                                               float ut, const float ud[3], float c00, float c01, float c11, float c22,
+                                               float c33) {
+    const float num = bsq + ph.cs2h * u, dn = rho + ph.wmph * u;
+    const float A = ut * ut * dn - num * c00;
+    const float c0[3] = {c01, 0.0f, 0.0f}, cd[3] = {c11, c22, c33};
+    const float idx[3] = {narrow(v.idx1), narrow(v.idx2), narrow(v.idx3)};
+    float sum = 0.0f;
+    bool ok = A > 1e-15f;
+#pragma unroll
+    for (int d = 0; d < 3; d++) {
+        const float B = ut * ud[d] * dn - num * c0[d];
+        const float C = ud[d] * ud[d] * dn - num * cd[d];
+        const float s = B * B - A * C;
+        sum += (fabsf(B) + (s > 0.0f ? sqrtf(s) : 0.0f)) * idx[d];
+        ok = ok && num * cd[d] > 1e-20f;
+    }
+    return ok ? sum / A : -1.0f;
+}
+// true where a rate of this estimate is certainly below the largest found so far (margin 1%)
+__device__ __forceinline__ bool rate_below(float est, const unsigned long long* dmax) {
+    const float cur = narrow(__longlong_as_double((long long)*(const volatile unsigned long long*)dmax));
+    return est >= 0.0f && est * 1.01f < cur;
+}
+// 2^(sh >> 20) brings the largest of three values to [1, 2) (0 where that is not above 2^-767)
+__device__ __forceinline__ int scale_of(double a, double b, double c) {
+    const int e = max(max(__double2hiint(a), __double2hiint(b)), __double2hiint(c)) & 0x7ff00000;
+    return e > 0x10000000 ? 0x3ff00000 - e : 0;
+}
+
+// largest of the warp's (non-negative) rates into *dmax
+__device__ __forceinline__ void reduce_rate(double inv, unsigned long long* dmax) {
+    const bool some = inv > 0.0;  // NaNs count as nothing
+    if (!__any_sync(0xffffffffu, some)) return;
+    unsigned long long b = some ? (unsigned long long)__double_as_longlong(inv) : 0ull;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long x = __shfl_xor_sync(0xffffffffu, b, o);
+        b = x > b ? x : b;
+    }
+    if ((threadIdx.x & 31u) == 0) atomicMax(dmax, b);
 }
 
 // Floors in the drift frame (Sec. 2.7, after Ressler et al. 2017): the floor
@@ -228,7 +291,9 @@ __device__ __forceinline__ bool drift_floor(const Metric<double>& m, const PhysA
     x[U3] = pa[U3];
     const double Bc[3] = {pr[B1], pr[B2], pr[B3]};
     int its = 0;
-    if (invert(U, Bc, m, gam, x, &its, false, nullptr, ph.inversion) == INV_FAIL) return false;
+    if (invert(U, Bc, m, gam, x, &its, false, nullptr, ph.inversion, ph.mixed ? C2P_NEWTON64 : C2P_NEWTON_FF) ==
+        INV_FAIL)
+        return false;
     pr[RHO] = fmax(x[RHO], rf);
     pr[UU] = fmax(x[UU], uf);
     pr[U1] = x[U1];
@@ -256,7 +321,7 @@ __device__ __forceinline__ int cell_floors(const BlockView& v, long g, const Met
     return 1;
 }
 
-// The same floors with b^2 given (the mixed-precision update takes it from its FP32 fluid
+// The same floors with b^2 given (the cell updates; the mixed-precision one takes it from its FP32 fluid
 // state); the drift frame forms the FP64 fluid state of pr where a floor applies.
 __device__ __forceinline__ int cell_floors_b2(const BlockView& v, long g, const Metric<double>& m, const PhysArgs& ph,
                                               double pr[NPRIM], double bsq) {
@@ -286,18 +351,11 @@ __device__ __forceinline__ void store_stage32(const BlockView& v, const PhysArgs
     if (corrector == 1) ph.un[(long)C_ENT * v.nc + c] = widen(kap);
 }
 
-// The floors of the mixed form in FP32: b^2 of the FP32 fluid state (like the fluxes), thresholds,
-// comparisons and floor values in FP32 (pf: the returned primitives rounded to FP32, updated with
-// pr); drift-frame floors take the FP64 path of cell_floors_b2
-__device__ __forceinline__ int cell_floors_f32(const BlockView& v, long g, const Metric<double>& m, const PhysArgs& ph,
-                                               double pr[NPRIM], float pf[NPRIM], float bsq) {
-    if (ph.floor_frame == HAMR_FLOOR_DRIFT) {
-        const int fl = cell_floors_b2(v, g, m, ph, pr, widen(bsq));
-        if (fl)
-#pragma unroll
-            for (int q = 0; q < NPRIM; q++) pf[q] = narrow(pr[q]);
-        return fl;
-    }
+// The fluid-frame floors of the mixed form in FP32: b^2 of the FP32 fluid state (like the fluxes),
+// thresholds, comparisons and floor values in FP32 (pf: the returned primitives rounded to FP32, updated
+// with pr)
+__device__ __forceinline__ int cell_floors_fluid32(const BlockView& v, long g, double pr[NPRIM], float pf[NPRIM],
+                                                   float bsq) {
     const float rf = fmaxf(narrow(v.gc[C_RHOFLR * v.n2d + g]), bsq * (1.0f / 50.0f));
     const float uf = fmaxf(narrow(v.gc[C_UFLR * v.n2d + g]), bsq * (1.0f / 750.0f));
     const bool lr = pf[RHO] < rf, lu = pf[UU] < uf;
@@ -311,6 +369,19 @@ __device__ __forceinline__ int cell_floors_f32(const BlockView& v, long g, const
         pr[UU] = widen(uf);
     }
     return 1;
+}
+
+// The same, or the drift frame's by the FP64 path of cell_floors_b2
+__device__ __forceinline__ int cell_floors_f32(const BlockView& v, long g, const Metric<double>& m, const PhysArgs& ph,
+                                               double pr[NPRIM], float pf[NPRIM], float bsq) {
+    if (ph.floor_frame == HAMR_FLOOR_DRIFT) {
+        const int fl = cell_floors_b2(v, g, m, ph, pr, widen(bsq));
+        if (fl)
+#pragma unroll
+            for (int q = 0; q < NPRIM; q++) pf[q] = narrow(pr[q]);
+        return fl;
+    }
+    return cell_floors_fluid32(v, g, pr, pf, bsq);
 }
 
 }  // namespace

@@ -536,8 +536,7 @@ struct WaveFF {
 template <int DIR>
 __device__ __forceinline__ WaveFF wave_ff(const PhysArgs& ph, double rho, double u, double bsq, double ut, double ud,
                                           ff c00, ff c0d, ff cdd) {
-    const int e = max(max(__double2hiint(rho), __double2hiint(u)), __double2hiint(bsq)) & 0x7ff00000;
-    const int sh = 0x3ff00000 - e;
+    const int sh = scale_of(rho, u, bsq);
     const ff R = ff_of(rho, sh), U = ff_of(u, sh), b = ff_of(bsq, sh), t = ff_of(ut), d = ff_of(ud);
     const ff num = ff_add(b, ff_mul(ff{ph.cs2h, ph.cs2l}, U));
     const ff dn = ff_add(R, ff_mul(ff{ph.wmph, ph.wmpl}, U));
@@ -890,6 +889,9 @@ __global__ void k_ct(BlockView v, const double* __restrict__ E, const double* Bb
 }
 
 
+// largest CFL rate of the block's cells. The FP64 rate of a cell is formed only where its FP32 estimate is
+// not certainly below the largest rate found so far (rate_below): in a spherical block nearly every cell is
+// (the largest rates sit next to the axis at the inner edge), and the result is the same bits.
 __device__ __forceinline__ void b_dt_reduce(const BlockView& v, PhysArgs ph, const double* __restrict__ P, unsigned long long* dmax, long t) {
     const long n = (long)v.n1 * v.n2 * v.n3;
     double inv = 0.0;
@@ -902,16 +904,27 @@ __device__ __forceinline__ void b_dt_reduce(const BlockView& v, PhysArgs ph, con
 #pragma unroll
         for (int q = 0; q < NPRIM; q++) pr[q] = P[q * v.nc + c];
         const int w = smr_width(v, ph, j);
-        if (w > 1) {  // an internal-SMR group: its width in x3
-            BlockView vw = v;
-            vw.idx3 = v.idx3 / w;
-            inv = inv_dt_cell(vw, pr, m, ph.gam);
-        } else {
-            inv = inv_dt_cell(v, pr, m, ph.gam);
-        }
+        BlockView vw = v;
+        if (w > 1) vw.idx3 = v.idx3 / w;  // an internal-SMR group: its width in x3
+        // the estimate's fluid state in FP32, (rho, u, B^2) scaled to O(1) by 2^sh, sh even
+        const int sh = scale_of(pr[RHO], pr[UU], 0.0) & ~0x100000;
+        Metric<float> mf;
+        mf.g01 = narrow(m.g01), mf.g03 = narrow(m.g03), mf.g11 = narrow(m.g11), mf.g13 = narrow(m.g13);
+        mf.g22 = narrow(m.g22), mf.g33 = narrow(m.g33);
+        const float q1 = narrow(pr[U1]), q2 = narrow(pr[U2]), q3 = narrow(pr[U3]);
+        const float u1 = mf.g11 * q1 + mf.g13 * q3, u2 = mf.g22 * q2, u3 = mf.g13 * q1 + mf.g33 * q3;
+        const float g2 = 1.0f + q1 * u1 + q2 * u2 + q3 * u3, gamma = sqrtf(g2);
+        const float al = narrow(m.alpha), c01 = narrow(m.c01);
+        const float b1 = ff_of(pr[B1], sh / 2).h, b2 = ff_of(pr[B2], sh / 2).h, b3 = ff_of(pr[B3], sh / 2).h;
+        const float bt = b1 * u1 + b2 * u2 + b3 * u3;
+        const float bb = mf.g11 * b1 * b1 + mf.g22 * b2 * b2 + mf.g33 * b3 * b3 + 2.0f * mf.g13 * b1 * b3;
+        const float bsq = al * al * (bb + bt * bt) / g2;
+        const float ud[3] = {q1 - gamma * al * c01, q2, q3};
+        const float est = rate_estimate(vw, ph, ff_of(pr[RHO], sh).h, ff_of(pr[UU], sh).h, bsq, gamma / al, ud,
+                                        narrow(m.c00), c01, narrow(m.c11), narrow(m.c22), narrow(m.c33));
+        if (!rate_below(est, dmax)) inv = inv_dt_cell(vw, pr, m, ph.gam);
     }
-    const double wmax = warp_max(inv);
-    if ((threadIdx.x & 31u) == 0 && wmax > 0.0) atomicMax(dmax, (unsigned long long)__double_as_longlong(wmax));
+    reduce_rate(inv, dmax);
 }
 
 __global__ void k_dt_reduce(BlockView v, PhysArgs ph, const double* __restrict__ P, unsigned long long* dmax) {
@@ -1068,7 +1081,8 @@ __global__ void k_reflux_cells(const DevBlock* tab, int n, const int* cblk, cons
     pr[B2] = Bc[1];
     pr[B3] = Bc[2];
     int its;
-    const int st = invert(U, Bc, m, ph.gam, pr, &its, false, nullptr, ph.inversion);
+    const int st = invert(U, Bc, m, ph.gam, pr, &its, false, nullptr, ph.inversion,
+                          ph.mixed ? C2P_NEWTON64 : C2P_NEWTON_FF);
     if (st == INV_FAIL)
 #pragma unroll
         for (int q = 0; q < 5; q++) pr[q] = D.P[q * v.nc + c];
@@ -1127,7 +1141,8 @@ __global__ void k_reflux_groups(const DevBlock* tab, int ngrp, const int* first,
     pr[B2] = Bc[1];
     pr[B3] = Bc[2];
     int its;
-    const int st = invert(U, Bc, m, ph.gam, pr, &its, false, nullptr, ph.inversion);
+    const int st = invert(U, Bc, m, ph.gam, pr, &its, false, nullptr, ph.inversion,
+                          ph.mixed ? C2P_NEWTON64 : C2P_NEWTON_FF);
     if (st == INV_FAIL)
 #pragma unroll
         for (int q = 0; q < 5; q++) pr[q] = p0[q];
@@ -1274,7 +1289,8 @@ __device__ __forceinline__ void b_smr_cells(const BlockView& v, const PhysArgs& 
     pr[B2] = Bc[1];
     pr[B3] = Bc[2];
     int its = 0;
-    const int st = invert(U, Bc, m, ph.gam, pr, &its, false, nullptr, ph.inversion);
+    const int st = invert(U, Bc, m, ph.gam, pr, &its, false, nullptr, ph.inversion,
+                          ph.mixed ? C2P_NEWTON64 : C2P_NEWTON_FF);
     if (st == INV_FAIL)
 #pragma unroll
         for (int q = 0; q < 5; q++) pr[q] = pf[q];
