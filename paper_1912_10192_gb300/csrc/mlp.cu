@@ -15,11 +15,16 @@
 namespace hamr {
 namespace {
 
-constexpr int TB = 128;  // samples (= threads) per CTA of the training kernels
-constexpr int HS = 65;   // row stride of the per-sample activation arrays (bank-conflict free)
-constexpr int XS = 11;   // row stride of the input array
-// shared memory of k_mlp_fb: parameters, inputs, three hidden layers, output errors
-constexpr int FB_SMEM = (MLP_NPARAM + 2 + TB * XS + 3 * TB * HS + TB * 2) * 4;
+constexpr int TB = 128;   // batches are multiples of this
+constexpr int TSMP = 64;  // samples per CTA of the training kernel
+constexpr int TTHR = 256; // its threads
+constexpr int HS = 68;    // row stride of its 64-wide arrays: 16-byte aligned rows, 16 bytes apart modulo the banks
+constexpr int XS = 12;    // row stride of its 10-wide arrays (two zeros)
+// shared memory of k_mlp_fb (floats): W2, W3, three hidden layers, W1, inputs, biases and W4, output errors
+constexpr int FB_W2 = 0, FB_W3 = 64 * HS, FB_H1 = 2 * 64 * HS, FB_H2 = FB_H1 + TSMP * HS, FB_H3 = FB_H2 + TSMP * HS,
+              FB_W1 = FB_H3 + TSMP * HS, FB_X = FB_W1 + 64 * XS, FB_B = FB_X + TSMP * XS, FB_W4 = FB_B + 192,
+              FB_B4 = FB_W4 + 128, FB_DY = FB_B4 + 4, FB_N = FB_DY + TSMP * 2;
+constexpr int FB_SMEM = FB_N * 4;
 
 __device__ __forceinline__ uint64_t splitmix64(uint64_t x) {  // Steele, Lea & Flood (2014)
     x += 0x9E3779B97F4A7C15ull;
@@ -140,147 +145,230 @@ __global__ void k_pack(const float* __restrict__ P, const float* __restrict__ no
 constexpr int PACK_THREADS = 64 * 16 + 2 * 4096 + IMGF_N;
 
 // ---------------------------------------------------------------- training (FP32)
-// One CTA: TB samples, forward and backward; the parameter gradient of
+// 64 x 64 products of a CTA's 64 samples, 256 threads with 4 x 4 results each in registers (tx = t & 15,
+// ty = t >> 4); operands in shared memory, read 16 bytes at a time without bank conflicts.
+
+// acc[r][q] += sum_i A[(ty + 16 r)][i] W[(tx + 16 q)][i], i < K (a multiple of 4)
+template <int K, int LD>
+__device__ __forceinline__ void mm_nt(const float* A, const float* W, int tx, int ty, float acc[4][4]) {
+#pragma unroll 4
+    for (int i = 0; i < K; i += 4) {
+        float4 a[4], w[4];
+#pragma unroll
+        for (int r = 0; r < 4; r++) a[r] = *reinterpret_cast<const float4*>(A + (ty + 16 * r) * LD + i);
+#pragma unroll
+        for (int q = 0; q < 4; q++) w[q] = *reinterpret_cast<const float4*>(W + (tx + 16 * q) * LD + i);
+#pragma unroll
+        for (int r = 0; r < 4; r++)
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                acc[r][q] = fmaf(a[r].x, w[q].x, acc[r][q]);
+                acc[r][q] = fmaf(a[r].y, w[q].y, acc[r][q]);
+                acc[r][q] = fmaf(a[r].z, w[q].z, acc[r][q]);
+                acc[r][q] = fmaf(a[r].w, w[q].w, acc[r][q]);
+            }
+    }
+}
+
+// one hidden layer: out[s][o] = tanh(b[o] + sum_i in[s][i] W[o][i])
+template <int K, int LD>
+__device__ __forceinline__ void mlp_layer(const float* in, const float* W, const float* b, float* out, int tx, int ty) {
+    float acc[4][4];
+#pragma unroll
+    for (int r = 0; r < 4; r++)
+#pragma unroll
+        for (int q = 0; q < 4; q++) acc[r][q] = b[tx + 16 * q];
+    mm_nt<K, LD>(in, W, tx, ty, acc);
+#pragma unroll
+    for (int r = 0; r < 4; r++)
+#pragma unroll
+        for (int q = 0; q < 4; q++) out[(ty + 16 * r) * HS + tx + 16 * q] = tanhf(acc[r][q]);
+}
+
+// One CTA: TSMP samples, forward and backward; the parameter gradient of
 // loss = sum over samples and outputs of r^2 / (2 count), r = yn - tn, is
 // accumulated into grad; sum r^2 into loss[0].
 // mode 0: samples off + 0.., mode 1: sample ids splitmix64(seed ^ (step * batch + b)) mod n.
-__global__ void __launch_bounds__(TB) k_mlp_fb(const float* __restrict__ Pg, const float* __restrict__ norm,
-                                               const float* __restrict__ feat, const float* __restrict__ targ,
-                                               int64_t n, int mode, int64_t off, int64_t count, uint64_t seed,
-                                               int64_t step, float* __restrict__ grad, float* __restrict__ loss) {
+// ~26000 FMAs per sample, latency-bound: a batch of 8192 took 104 us with one thread per sample (two shared
+// loads per FMA, 64 CTAs of 4 warps), 24 us with register tiles (128 CTAs of 8 warps).
+__global__ void __launch_bounds__(TTHR) k_mlp_fb(const float* __restrict__ Pg, const float* __restrict__ norm,
+                                                 const float* __restrict__ feat, const float* __restrict__ targ,
+                                                 int64_t n, int mode, int64_t off, int64_t count, uint64_t seed,
+                                                 int64_t step, float* __restrict__ grad, float* __restrict__ loss) {
     extern __shared__ __align__(16) float fsm[];
-    float* P = fsm;                       // MLP_NPARAM (+2 pad)
-    float* X = P + MLP_NPARAM + 2;        // TB x XS
-    float* H1 = X + TB * XS;              // TB x HS, later dz1
-    float* H2 = H1 + TB * HS;             // later dz2
-    float* H3 = H2 + TB * HS;             // later dz3
-    float* DY = H3 + TB * HS;             // TB x 2
-    const int t = threadIdx.x;
-    for (int q = t; q < MLP_NPARAM; q += TB) P[q] = Pg[q];
-    const int64_t b = (int64_t)blockIdx.x * TB + t;
-    int64_t g = 0;
-    bool active;
-    if (mode == 0) {
-        g = off + b;
-        active = (b < count) && (g < n);
-    } else {
-        active = b < count;
+    float *W2 = fsm + FB_W2, *W3 = fsm + FB_W3, *H1 = fsm + FB_H1, *H2 = fsm + FB_H2, *H3 = fsm + FB_H3;
+    float *W1 = fsm + FB_W1, *X = fsm + FB_X, *Bs = fsm + FB_B, *W4 = fsm + FB_W4, *B4 = fsm + FB_B4, *DY = fsm + FB_DY;
+    const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
+    auto sample = [&](int s, int64_t& g) {  // whether sample s of the CTA counts, and its row
+        const int64_t b = (int64_t)blockIdx.x * TSMP + s;
+        if (mode == 0) {
+            g = off + b;
+            return (b < count) && (g < n);
+        }
         g = (int64_t)(splitmix64(seed ^ (uint64_t)(step * count + b)) % (uint64_t)n);
+        return b < count;
+    };
+#pragma unroll
+    for (int q = 0; q < 4; q++) {  // 1024 float4 of W2 and of W3
+        const int e = t + TTHR * q, o = e >> 4, i = (e & 15) * 4;
+        *reinterpret_cast<float4*>(W2 + o * HS + i) = *reinterpret_cast<const float4*>(Pg + P_W2 + o * 64 + i);
+        *reinterpret_cast<float4*>(W3 + o * HS + i) = *reinterpret_cast<const float4*>(Pg + P_W3 + o * 64 + i);
     }
-    const float* W1 = P + P_W1;
-    const float* W2 = P + P_W2;
-    const float* W3 = P + P_W3;
-    const float* W4 = P + P_W4;
+    for (int e = t; e < 64 * XS; e += TTHR) {
+        const int o = e / XS, i = e % XS;
+        W1[e] = i < MLP_NIN ? Pg[P_W1 + o * MLP_NIN + i] : 0.0f;
+    }
+    if (t < 64) {
+        Bs[t] = Pg[P_B1 + t];
+        Bs[64 + t] = Pg[P_B2 + t];
+        Bs[128 + t] = Pg[P_B3 + t];
+    } else if (t < 192) {
+        W4[t - 64] = Pg[P_W4 + t - 64];
+    } else if (t < 194) {
+        B4[t - 192] = Pg[P_B4 + t - 192];
+    }
+    {
+        const int s = t & 63;
+        int64_t g;
+        const bool on = sample(s, g);
+        for (int i = t >> 6; i < XS; i += 4)
+            X[s * XS + i] = (on && i < MLP_NIN) ? (feat[i * n + g] - norm[i]) / norm[10 + i] : 0.0f;
+    }
     __syncthreads();
     // forward
-    float x[MLP_NIN];
-#pragma unroll
-    for (int i = 0; i < MLP_NIN; i++) {
-        x[i] = active ? (feat[i * n + g] - norm[i]) / norm[10 + i] : 0.0f;
-        X[t * XS + i] = x[i];
-    }
-    for (int o = 0; o < 64; o++) {
-        float z = P[P_B1 + o];
-#pragma unroll
-        for (int i = 0; i < MLP_NIN; i++) z = fmaf(W1[o * MLP_NIN + i], x[i], z);
-        H1[t * HS + o] = tanhf(z);
-    }
-    for (int o = 0; o < 64; o++) {
-        float z = P[P_B2 + o];
-        for (int i = 0; i < 64; i++) z = fmaf(W2[o * 64 + i], H1[t * HS + i], z);
-        H2[t * HS + o] = tanhf(z);
-    }
-    for (int o = 0; o < 64; o++) {
-        float z = P[P_B3 + o];
-        for (int i = 0; i < 64; i++) z = fmaf(W3[o * 64 + i], H2[t * HS + i], z);
-        H3[t * HS + o] = tanhf(z);
-    }
+    mlp_layer<XS, XS>(X, W1, Bs, H1, tx, ty);
+    __syncthreads();
+    mlp_layer<64, HS>(H1, W2, Bs + 64, H2, tx, ty);
+    __syncthreads();
+    mlp_layer<64, HS>(H2, W3, Bs + 128, H3, tx, ty);
+    __syncthreads();
     float r2 = 0.0f;
-    const float inv_count = 1.0f / (float)count;
-#pragma unroll
-    for (int j = 0; j < 2; j++) {
-        float y = P[P_B4 + j];
-        for (int o = 0; o < 64; o++) y = fmaf(W4[j * 64 + o], H3[t * HS + o], y);
-        const float tn = active ? (targ[j * n + g] - norm[20 + j]) / norm[22 + j] : 0.0f;
-        const float r = active ? y - tn : 0.0f;
-        r2 += r * r;
-        DY[t * 2 + j] = r * inv_count;
+    if (t < 2 * TSMP) {
+        const int s = t >> 1, j = t & 1;
+        int64_t g;
+        const bool on = sample(s, g);
+        float y = B4[j];
+        for (int o = 0; o < 64; o += 4) {
+            const float4 h = *reinterpret_cast<const float4*>(H3 + s * HS + o);
+            const float4 w = *reinterpret_cast<const float4*>(W4 + j * 64 + o);
+            y = fmaf(w.x, h.x, y);
+            y = fmaf(w.y, h.y, y);
+            y = fmaf(w.z, h.z, y);
+            y = fmaf(w.w, h.w, y);
+        }
+        const float r = on ? y - (targ[j * n + g] - norm[20 + j]) / norm[22 + j] : 0.0f;
+        r2 = r * r;
+        DY[s * 2 + j] = r * (1.0f / (float)count);
     }
     __syncthreads();
-    // output layer gradients
+    // output layer gradients: (j, o) over half the samples each
     {
-        const int j = t >> 6, o = t & 63;
+        const int o = t & 63, j = (t >> 6) & 1, s0 = (t >> 7) * (TSMP / 2);
         float a = 0.0f;
-        for (int s = 0; s < TB; s++) a = fmaf(DY[s * 2 + j], H3[s * HS + o], a);
+        for (int s = s0; s < s0 + TSMP / 2; s++) a = fmaf(DY[s * 2 + j], H3[s * HS + o], a);
         atomicAdd(&grad[P_W4 + j * 64 + o], a);
         if (t < 2) {
             float bsum = 0.0f;
-            for (int s = 0; s < TB; s++) bsum += DY[s * 2 + t];
+            for (int s = 0; s < TSMP; s++) bsum += DY[s * 2 + t];
             atomicAdd(&grad[P_B4 + t], bsum);
         }
     }
     __syncthreads();
-    // dz3 = (W4^T dy) (1 - h3^2), own row
-    for (int o = 0; o < 64; o++) {
-        const float h = H3[t * HS + o];
-        H3[t * HS + o] = (W4[o] * DY[t * 2] + W4[64 + o] * DY[t * 2 + 1]) * (1.0f - h * h);
+    // dz3 = (W4^T dy) (1 - h3^2)
+    {
+        const int o = t & 63;
+        for (int s = t >> 6; s < TSMP; s += 4) {
+            const float h = H3[s * HS + o];
+            H3[s * HS + o] = (W4[o] * DY[s * 2] + W4[64 + o] * DY[s * 2 + 1]) * (1.0f - h * h);
+        }
     }
     __syncthreads();
     // hidden layers 3 and 2: dW = dz^T h_prev, db = sum dz; then dz_prev = (W^T dz) (1 - h_prev^2)
 #pragma unroll 1
     for (int layer = 3; layer >= 2; layer--) {
-        float* Z = (layer == 3) ? H3 : H2;
+        const float* Z = (layer == 3) ? H3 : H2;
         float* Hp = (layer == 3) ? H2 : H1;
         const float* Wl = (layer == 3) ? W3 : W2;
         const int pw = (layer == 3) ? P_W3 : P_W2, pb = (layer == 3) ? P_B3 : P_B2;
-        {
-            const int o = t >> 1, i0 = (t & 1) * 32;
-            float acc[32];
+        float acc[4][4];
 #pragma unroll
-            for (int q = 0; q < 32; q++) acc[q] = 0.0f;
-            float bs = 0.0f;
-            for (int s = 0; s < TB; s++) {
-                const float z = Z[s * HS + o];
-                bs += z;
+        for (int r = 0; r < 4; r++)
 #pragma unroll
-                for (int q = 0; q < 32; q++) acc[q] = fmaf(z, Hp[s * HS + i0 + q], acc[q]);
-            }
+            for (int q = 0; q < 4; q++) acc[r][q] = 0.0f;
+#pragma unroll 4
+        for (int s = 0; s < TSMP; s++) {  // outputs 4 ty + r, inputs 4 tx + q
+            const float4 z = *reinterpret_cast<const float4*>(Z + s * HS + 4 * ty);
+            const float4 h = *reinterpret_cast<const float4*>(Hp + s * HS + 4 * tx);
+            const float zr[4] = {z.x, z.y, z.z, z.w}, hq[4] = {h.x, h.y, h.z, h.w};
 #pragma unroll
-            for (int q = 0; q < 32; q++) atomicAdd(&grad[pw + o * 64 + i0 + q], acc[q]);
-            if ((t & 1) == 0) atomicAdd(&grad[pb + o], bs);
+            for (int r = 0; r < 4; r++)
+#pragma unroll
+                for (int q = 0; q < 4; q++) acc[r][q] = fmaf(zr[r], hq[q], acc[r][q]);
         }
-        __syncthreads();
-        {
-            float dz[64];
-            for (int i = 0; i < 64; i++) {
-                float a = 0.0f;
-                for (int o = 0; o < 64; o++) a = fmaf(Wl[o * 64 + i], Z[t * HS + o], a);
-                const float h = Hp[t * HS + i];
-                dz[i] = a * (1.0f - h * h);
+#pragma unroll
+        for (int r = 0; r < 4; r++) {  // pairs: the gradient's base is 8-byte aligned
+            float2* g = reinterpret_cast<float2*>(grad + pw + (4 * ty + r) * 64 + 4 * tx);
+            atomicAdd(g, make_float2(acc[r][0], acc[r][1]));
+            atomicAdd(g + 1, make_float2(acc[r][2], acc[r][3]));
+        }
+        if (t < 64) {
+            float bs = 0.0f;
+            for (int s = 0; s < TSMP; s++) bs += Z[s * HS + t];
+            atomicAdd(&grad[pb + t], bs);
+        }
+#pragma unroll
+        for (int r = 0; r < 4; r++)
+#pragma unroll
+            for (int q = 0; q < 4; q++) acc[r][q] = 0.0f;
+#pragma unroll 4
+        for (int o = 0; o < 64; o += 4) {  // samples ty + 16 r, inputs 4 tx + q
+            float4 z[4], w[4];
+#pragma unroll
+            for (int r = 0; r < 4; r++) z[r] = *reinterpret_cast<const float4*>(Z + (ty + 16 * r) * HS + o);
+#pragma unroll
+            for (int u = 0; u < 4; u++) w[u] = *reinterpret_cast<const float4*>(Wl + (o + u) * HS + 4 * tx);
+#pragma unroll
+            for (int r = 0; r < 4; r++) {
+                const float zu[4] = {z[r].x, z[r].y, z[r].z, z[r].w};
+#pragma unroll
+                for (int u = 0; u < 4; u++) {
+                    acc[r][0] = fmaf(zu[u], w[u].x, acc[r][0]);
+                    acc[r][1] = fmaf(zu[u], w[u].y, acc[r][1]);
+                    acc[r][2] = fmaf(zu[u], w[u].z, acc[r][2]);
+                    acc[r][3] = fmaf(zu[u], w[u].w, acc[r][3]);
+                }
             }
-            for (int i = 0; i < 64; i++) Hp[t * HS + i] = dz[i];
+        }
+        __syncthreads();  // every thread has read h_prev
+#pragma unroll
+        for (int r = 0; r < 4; r++) {
+            float4* d = reinterpret_cast<float4*>(Hp + (ty + 16 * r) * HS + 4 * tx);
+            const float4 h = *d;
+            *d = make_float4(acc[r][0] * (1.0f - h.x * h.x), acc[r][1] * (1.0f - h.y * h.y),
+                             acc[r][2] * (1.0f - h.z * h.z), acc[r][3] * (1.0f - h.w * h.w));
         }
         __syncthreads();
     }
-    // first layer: dW1 = dz1^T x, db1
+    // first layer: dW1 = dz1^T x (three of the twelve columns per thread), db1
     {
-        const int o = t >> 1, i0 = (t & 1) * 5;
-        float acc[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+        const int o = t >> 2, i0 = (t & 3) * 3;
+        float acc[3] = {0.0f, 0.0f, 0.0f};
         float bs = 0.0f;
-        for (int s = 0; s < TB; s++) {
+        for (int s = 0; s < TSMP; s++) {
             const float z = H1[s * HS + o];
             bs += z;
 #pragma unroll
-            for (int q = 0; q < 5; q++) acc[q] = fmaf(z, X[s * XS + i0 + q], acc[q]);
+            for (int q = 0; q < 3; q++) acc[q] = fmaf(z, X[s * XS + i0 + q], acc[q]);
         }
 #pragma unroll
-        for (int q = 0; q < 5; q++) atomicAdd(&grad[P_W1 + o * MLP_NIN + i0 + q], acc[q]);
-        if ((t & 1) == 0) atomicAdd(&grad[P_B1 + o], bs);
+        for (int q = 0; q < 3; q++)
+            if (i0 + q < MLP_NIN) atomicAdd(&grad[P_W1 + o * MLP_NIN + i0 + q], acc[q]);
+        if ((t & 3) == 0) atomicAdd(&grad[P_B1 + o], bs);
     }
     // loss
     float v = r2;
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((t & 31) == 0) atomicAdd(loss, v);
+    if ((t & 31) == 0 && t < 2 * TSMP) atomicAdd(loss, v);
 }
 
 __global__ void k_adam(float* __restrict__ P, float* __restrict__ grad, float* __restrict__ m1,
@@ -535,9 +623,9 @@ int hamr_mlp_train(hamr_mlp* m, int64_t n, const float* feat, const float* targ,
     MLP_CUDA(cudaFuncSetAttribute(k_mlp_fb, cudaFuncAttributeMaxDynamicSharedMemorySize, FB_SMEM));
     MLP_CUDA(cudaMemsetAsync(m->loss, 0, (size_t)a->steps * sizeof(float), s));
     MLP_CUDA(cudaMemsetAsync(m->grad, 0, MLP_NPARAM * sizeof(float), s));
-    const unsigned nb = (unsigned)(a->batch / TB);
+    const unsigned nb = (unsigned)(a->batch / TSMP);
     for (int64_t k = 0; k < a->steps; k++) {
-        k_mlp_fb<<<nb, TB, FB_SMEM, s>>>(m->params, m->norm, feat, targ, n, 1, 0, a->batch, a->seed, k, m->grad,
+        k_mlp_fb<<<nb, TTHR, FB_SMEM, s>>>(m->params, m->norm, feat, targ, n, 1, 0, a->batch, a->seed, k, m->grad,
                                          m->loss + k);
         m->adam_t++;
         const double tt = (double)m->adam_t;
@@ -570,8 +658,8 @@ int hamr_mlp_loss_grad(hamr_mlp* m, int64_t n, const float* feat, const float* t
     MLP_CUDA(cudaFuncSetAttribute(k_mlp_fb, cudaFuncAttributeMaxDynamicSharedMemorySize, FB_SMEM));
     MLP_CUDA(cudaMemsetAsync(m->loss, 0, sizeof(float), s));
     MLP_CUDA(cudaMemsetAsync(m->grad, 0, MLP_NPARAM * sizeof(float), s));
-    const unsigned nb = (unsigned)((n + TB - 1) / TB);
-    k_mlp_fb<<<nb, TB, FB_SMEM, s>>>(m->params, m->norm, feat, targ, n, 0, 0, n, 0, 0, m->grad, m->loss);
+    const unsigned nb = (unsigned)((n + TSMP - 1) / TSMP);
+    k_mlp_fb<<<nb, TTHR, FB_SMEM, s>>>(m->params, m->norm, feat, targ, n, 0, 0, n, 0, 0, m->grad, m->loss);
     MLP_CUDA(cudaGetLastError());
     MLP_CUDA(cudaMemcpyAsync(grad, m->grad, MLP_NPARAM * sizeof(float), cudaMemcpyDeviceToHost, s));
     MLP_CUDA(cudaMemcpyAsync(loss, m->loss, sizeof(float), cudaMemcpyDeviceToHost, s));
