@@ -1710,6 +1710,11 @@ int amr_create(AmrImpl** out, const hamr_grid_desc& d, const std::vector<BlockVi
 
 void amr_destroy(AmrImpl* M) { delete M; }
 
+void amr_old_state(const AmrImpl* M, int b, double** Pold, double** Bold) {
+    *Pold = M->H.b[b].Pold;
+    *Bold = M->H.b[b].Bold;
+}
+
 int amr_after_load(AmrImpl* M, int b, cudaStream_t s) {
     // no history yet: the previous state is the loaded one
     const DevBlock& D = M->H.b[b];

@@ -374,6 +374,18 @@ int copy_fields(double* dst, long dstride, const double* src, long sstride, long
     return HAMR_OK;
 }
 
+// Whether a kernel on the grid's device can take the pointer: memory of that device, or managed. Other
+// pointers (another device's, page-locked or plain host memory) go through the runtime's copies, which take
+// what they can and refuse the rest.
+bool kernel_can_reach(const hamr_grid* g, const void* p) {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return (a.type == cudaMemoryTypeDevice && a.device == g->device) || a.type == cudaMemoryTypeManaged;
+}
+
 int check_block(const hamr_grid* g, int block) {
     if (!g) return fail(HAMR_EINVAL, "grid is NULL");
     if (block < 0 || block >= (int)g->blocks.size()) return fail(HAMR_EINVAL, "block %d out of range", block);
@@ -463,6 +475,18 @@ int hamr_grid_set_state(hamr_grid* g, int block, const double* prim, const doubl
     const BlockView& v = g->view[block];
     BlockState& s = g->st[block];
     const long n = (long)v.n1p * v.n2p * v.n3p;
+    if (on_device && kernel_can_reach(g, prim) && kernel_can_reach(g, bface)) {
+        cudaStream_t cs = S(stream);
+        double *Po = nullptr, *Bo = nullptr;
+        if (g->amr) amr_old_state(g->amr, block, &Po, &Bo);  // no history yet: the previous state is the loaded one
+        CUDA_TRY(cudaMemsetAsync(s.dmax, 0, sizeof(unsigned long long), cs));
+        LAUNCH(g, K_LOAD, 1, cs, launch_load(v, g->ph, prim, bface, s.P, s.B, Po, Bo, s.dmax, cs));
+        if (!g->amr) LAUNCH(g, K_LOAD, 1, cs, launch_bc(v, s.P, s.B, cs));
+        g->stage32_valid = false;
+        g->ghosts_valid = (g->amr == nullptr);
+        g->loaded[block] = 1;
+        return HAMR_OK;
+    }
     const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     rc = copy_fields(s.P, v.nc, prim, n, n, 8, kind, S(stream), !on_device);
     if (rc) return rc;
@@ -470,7 +494,7 @@ int hamr_grid_set_state(hamr_grid* g, int block, const double* prim, const doubl
     if (rc) return rc;
     cudaStream_t cs = S(stream);
     CUDA_TRY(cudaMemsetAsync(s.dmax, 0, sizeof(unsigned long long), cs));
-    LAUNCH(g, K_LOAD, g->amr ? 2 : 6, cs, load_kernels(v, g->ph, s, g->amr == nullptr, cs));
+    LAUNCH(g, K_LOAD, g->amr ? 2 : 3, cs, load_kernels(v, g->ph, s, g->amr == nullptr, cs));
     g->stage32_valid = false;
     g->ghosts_valid = (g->amr == nullptr);  // the load applied the boundary conditions
     if (g->amr) {
@@ -487,6 +511,10 @@ int hamr_grid_get_state(const hamr_grid* g, int block, double* prim, double* bfa
     const BlockView& v = g->view[block];
     const BlockState& s = g->st[block];
     const long n = (long)v.n1p * v.n2p * v.n3p;
+    if (on_device && (prim || bface) && (!prim || kernel_can_reach(g, prim)) && (!bface || kernel_can_reach(g, bface))) {
+        CUDA_TRY(launch_store(v, s.P, s.B, prim, bface, S(stream)));
+        return HAMR_OK;
+    }
     if (!on_device) CUDA_TRY(cudaStreamSynchronize(S(stream)));
     const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
     if (prim) {
@@ -518,7 +546,7 @@ int hamr_block_step(hamr_grid* g, int block, double dt, void* stream, hamr_step_
     const bool fused = ph.stage32 && g->stage32_valid;
     // predictor: P^n, B^n -> P^{n+1/2}, B^{n+1/2} (the ghosts of P^n are current after a load or a step,
     // which end with the boundary conditions)
-    if (!g->ghosts_valid) LAUNCH(g, K_BC, 4, cs, launch_bc(v, s.P, s.B, cs, P32g, K32g));
+    if (!g->ghosts_valid) LAUNCH(g, K_BC, 1, cs, launch_bc(v, s.P, s.B, cs, P32g, K32g));
     g->ghosts_valid = false;  // until this step has ended (an error on the way leaves them unknown)
     g->stage32_valid = false;
     if (ph.mixed && !fused) LAUNCH(g, K_BC, 1, cs, launch_to_f32(v, s.P, s.P32, cs));
@@ -536,7 +564,7 @@ int hamr_block_step(hamr_grid* g, int block, double dt, void* stream, hamr_step_
     if (ph.smr)
         LAUNCH(g, K_UPDATE, 1, cs, launch_smr_cells(v, ph, 0, s.P, s.Bh, s.Ph, s.status, s.dmax, s.dcnt, cs));
     // corrector: U^n and the fluxes of P^{n+1/2} -> P^{n+1}, B^{n+1} (in place)
-    LAUNCH(g, K_BC, 4, cs, launch_bc(v, s.Ph, s.Bh, cs, P32g, K32g));
+    LAUNCH(g, K_BC, 1, cs, launch_bc(v, s.Ph, s.Bh, cs, P32g, K32g));
     if (ph.mixed && !ph.stage32) LAUNCH(g, K_BC, 1, cs, launch_to_f32(v, s.Ph, s.P32, cs));
     if (!ph.stage32) LAUNCH(g, K_RECON, 1, cs, launch_kappa(v, ph, s.Ph, s.P32, s.E, nullptr, cs));
     for (int dir = 1; dir <= 3; dir++) {
@@ -551,7 +579,7 @@ int hamr_block_step(hamr_grid* g, int block, double dt, void* stream, hamr_step_
            launch_update(v, ph, 1, s.Ph, s.F, s.B, s.Un, s.P, s.status, s.dscal, 1.0, s.dmax, s.dcnt, cs));
     if (ph.smr)
         LAUNCH(g, K_UPDATE, 1, cs, launch_smr_cells(v, ph, 1, s.Ph, s.B, s.P, s.status, s.dmax, s.dcnt, cs));
-    LAUNCH(g, K_BC, 4, cs, launch_bc(v, s.P, s.B, cs, P32g, K32g));
+    LAUNCH(g, K_BC, 1, cs, launch_bc(v, s.P, s.B, cs, P32g, K32g));
     g->stage32_valid = ph.stage32 != 0;
     g->ghosts_valid = true;
     if (stats) {
@@ -586,7 +614,7 @@ int hamr_grid_fill_ghosts(hamr_grid* g, void* stream) {
     for (size_t b = 0; b < g->loaded.size(); b++)
         if (!g->loaded[b]) return fail(HAMR_ESTATE, "block %zu has no state", b);
     if (g->amr) return amr_fill(g->amr, S(stream));
-    LAUNCH(g, K_BC, 4, S(stream), launch_bc(g->view[0], g->st[0].P, g->st[0].B, S(stream)));
+    LAUNCH(g, K_BC, 1, S(stream), launch_bc(g->view[0], g->st[0].P, g->st[0].B, S(stream)));
     return HAMR_OK;
 }
 

@@ -218,6 +218,12 @@ cudaError_t launch_centre_b(const BlockView& v, double* P, const double* B, cuda
 cudaError_t launch_block_max(const BlockView& v, const double* P, int q, unsigned long long* out, cudaStream_t s);
 cudaError_t launch_bc(const BlockView& v, double* P, double* B, cudaStream_t s, float* P32 = nullptr,
                       float* K32 = nullptr);
+// a whole state between the caller's device arrays (field stride: the padded cell count) and the block:
+// in with the centre field and the CFL rate, Po, Bo: a tree's old state (or null); out: prim, bface may be null
+cudaError_t launch_load(const BlockView& v, const PhysArgs& ph, const double* prim, const double* bface, double* P,
+                        double* B, double* Po, double* Bo, unsigned long long* dmax, cudaStream_t s);
+cudaError_t launch_store(const BlockView& v, const double* P, const double* B, double* prim, double* bface,
+                         cudaStream_t s);
 // entropy tracer kappa = p / rho^gam of every padded cell into K (FP32 view of K when mixed)
 // Un: the U^n cache (predictor) or nullptr (corrector); the predictor stores kappa in its entropy slot
 cudaError_t launch_kappa(const BlockView& v, const PhysArgs& ph, const double* P, const float* P32, double* K,
@@ -328,6 +334,7 @@ int amr_create(AmrImpl** out, const hamr_grid_desc& d, const std::vector<BlockVi
                const std::vector<BlockState>& st, const PhysArgs& ph);
 void amr_destroy(AmrImpl* M);
 int amr_after_load(AmrImpl* M, int block, cudaStream_t s);
+void amr_old_state(const AmrImpl* M, int block, double** Pold, double** Bold);
 int amr_period(AmrImpl* M, cudaStream_t s, int nperiods, bool use_graph);
 int amr_info(const AmrImpl* M, int* lmax, double* dtf_host);
 int amr_links(const AmrImpl* M, int* counts5);

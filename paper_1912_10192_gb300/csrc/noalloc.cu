@@ -189,8 +189,7 @@ extern "C" int hamr_block_step_noalloc(const hamr_grid_desc* d, double* prim, do
     NA_TRY(launch_bc(v, s.P, s.B, cs));
     NA_TRY(launch_dt_reduce(v, ph, s.P, s.dmax, cs));
     NA_TRY(launch_dt_select(ph, dt, s.dscal, s.dmax, s.dcnt, s.status, v.nc, cs));
-    // predictor
-    NA_TRY(launch_bc(v, s.P, s.B, cs));
+    // predictor (the ghosts are the load's)
     NA_TRY(launch_kappa(v, ph, s.P, nullptr, s.E, s.Un, cs));
     for (int dir = 1; dir <= 3; dir++) {
         if (ph.flatten) NA_TRY(launch_flatten(v, ph, dir, s.P, nullptr, s.F[dir - 1], cs));

@@ -22,13 +22,16 @@ inline unsigned nblk(long n, int bs = BS) { return (unsigned)((n + bs - 1) / bs)
 
 // ---------------------------------------------------------------- centre B
 // B^i = (Bbar^i_lo + Bbar^i_hi) / 2 / sqrt(-g)_centre (Sec. 2.5)
-__device__ __forceinline__ void centre_field(const BlockView& v, const double* __restrict__ B, int i, int j, int k,
-                                             double ig, double Bc[3]) {  // ig = 1 / sqrt(-g)
-    const long c = cidx(v, i, j, k);
+__device__ __forceinline__ void centre_field_at(const BlockView& v, const double* __restrict__ B, long stride, long c,
+                                                double ig, double Bc[3]) {  // ig = 1 / sqrt(-g)
     const double hig = 0.5 * ig;
     Bc[0] = (B[c] + B[c + 1]) * hig;
-    Bc[1] = (B[v.nc + c] + B[v.nc + c + v.n1p]) * hig;
-    Bc[2] = (B[2 * v.nc + c] + B[2 * v.nc + c + (long)v.n1p * v.n2p]) * hig;
+    Bc[1] = (B[stride + c] + B[stride + c + v.n1p]) * hig;
+    Bc[2] = (B[2 * stride + c] + B[2 * stride + c + (long)v.n1p * v.n2p]) * hig;
+}
+__device__ __forceinline__ void centre_field(const BlockView& v, const double* __restrict__ B, int i, int j, int k,
+                                             double ig, double Bc[3]) {
+    centre_field_at(v, B, v.nc, cidx(v, i, j, k), ig, Bc);
 }
 
 __device__ __forceinline__ long tidx() { return (long)blockIdx.x * blockDim.x + threadIdx.x; }

@@ -30,11 +30,11 @@ __global__ void k_centre_b(BlockView v, double* __restrict__ P, const double* __
 
 
 // ---------------------------------------------------------------- boundaries
-// One pass per direction e, in the order x3, x2, x1, each over the full
-// padded extent of the other two directions. Polar (x2): ghost (j = -1-m, k)
-// takes (j = m, k + n3/2) with utilde^2, B^2 and Bbar^2 negated; axis faces 0.
-// Outflow: copy of the last interior cell/face; NOINFLOW clamps utilde^1.
-// Periodic: wrap; face n takes face 0.
+// The conditions of x3, x2, x1 in this order, each over the full padded extent of the other two
+// directions, composed: a ghost cell takes the interior cell that its x1, then x2, then x3 map lead to.
+// Polar (x2): ghost (j = -1-m, k) takes (j = m, k + n3/2) with utilde^2, B^2 and Bbar^2 negated; axis
+// faces 0. Outflow: copy of the last interior cell/face; NOINFLOW clamps utilde^1. Periodic: wrap; face n
+// takes face 0.
 __device__ __forceinline__ int cell_src(int bc, int n, int g) {
     if (bc == HAMR_BC_PERIODIC) return g < 0 ? g + n : g - n;
     if (bc == HAMR_BC_POLAR) return g < 0 ? -1 - g : 2 * n - 1 - g;
@@ -46,68 +46,88 @@ __device__ __forceinline__ int face_src(int bc, int n, int g) {
     return g < 0 ? 0 : n;
 }
 
-// P32, K32 (mixed precision on a single block, else null): the ghost cells of the FP32 copy of the
-// primitives and of its entropy tracer kappa, from the same sources
-__global__ void k_bc_pass(BlockView v, double* __restrict__ P, double* __restrict__ B, int e, float* __restrict__ P32,
-                          float* __restrict__ K32) {
-    const int nn[4] = {0, v.n1, v.n2, v.n3};
-    const int ta = (e == 1) ? 2 : 1, tb = (e == 3) ? 2 : 3;
-    const int na = nn[ta] + 2 * NG, nb = nn[tb] + 2 * NG;
-    const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long total = 2L * NG * na * nb;
-    if (t >= total) return;
-    const int a = (int)(t % na) - NG;
-    const int b = (int)((t / na) % nb) - NG;
-    const int m = (int)((t / ((long)na * nb)) % NG);
-    const int side = (int)(t / ((long)na * nb * NG));
-    const int bc = v.bc[2 * (e - 1) + side];
-    const bool polar = (bc == HAMR_BC_POLAR);
-    int ss[4] = {0, 0, 0, 0}, dd[4] = {0, 0, 0, 0};
-    ss[ta] = a;
-    ss[tb] = b;
-    if (polar) ss[3] = ((b + v.n3 / 2) % v.n3 + v.n3) % v.n3;
-    dd[ta] = a;
-    dd[tb] = b;
-    const int gi = (side == 0) ? -1 - m : nn[e] + m;
-    dd[e] = gi;
-    ss[e] = cell_src(bc, nn[e], gi);
-    long dst = cidx(v, dd[1], dd[2], dd[3]), src = cidx(v, ss[1], ss[2], ss[3]);
+// the interior location that (x[1], x[2], x[3]) takes its value from, in place; f: the direction of a face
+// field's component (0: a cell field). Returns whether a polar map was passed.
+__device__ __forceinline__ bool bc_source(const BlockView& v, int f, int x[4]) {
+    const int n[4] = {0, v.n1, v.n2, v.n3};
+    bool polar = false;
 #pragma unroll
-    for (int q = 0; q < NPRIM; q++) {
-        double x = P[q * v.nc + src];
-        if (polar && (q == U2 || q == B2)) x = -x;
-        if (q == U1 && bc == HAMR_BC_OUTFLOW_NOINFLOW && e == 1) {
-            if (side == 1 && x < 0.0) x = 0.0;
-            if (side == 0 && x > 0.0) x = 0.0;
+    for (int e = 1; e <= 3; e++) {
+        const int hi = n[e] + ((f == e && v.bc[2 * e - 1] != HAMR_BC_PERIODIC) ? 1 : 0);  // first ghost above
+        if (x[e] >= 0 && x[e] < hi) continue;
+        const int bc = v.bc[2 * (e - 1) + (x[e] < 0 ? 0 : 1)];
+        x[e] = (f == e) ? face_src(bc, n[e], x[e]) : cell_src(bc, n[e], x[e]);
+        if (bc == HAMR_BC_POLAR) {
+            polar = true;
+            x[3] = ((x[3] + v.n3 / 2) % v.n3 + v.n3) % v.n3;
         }
-        P[q * v.nc + dst] = x;
-        if (P32) P32[q * v.nc + dst] = (float)x;
     }
-    if (K32) K32[dst] = K32[src];  // kappa depends on rho and u only, which the map keeps
-#pragma unroll
-    for (int f = 1; f <= 3; f++)
-        if (f != e) B[(f - 1) * v.nc + dst] = B[(f - 1) * v.nc + src];
-    const int gf = (side == 0) ? -1 - m : nn[e] + (bc == HAMR_BC_PERIODIC ? 0 : 1) + m;
-    if (gf < nn[e] + NG) {
-        dd[e] = gf;
-        ss[e] = face_src(bc, nn[e], gf);
-        dst = cidx(v, dd[1], dd[2], dd[3]);
-        src = cidx(v, ss[1], ss[2], ss[3]);
-        const double x = B[(e - 1) * v.nc + src];
-        B[(e - 1) * v.nc + dst] = polar ? -x : x;
-    }
+    return polar;
 }
 
-// axis faces hold 0 (after the x2 pass wrote its ghosts)
-__global__ void k_bc_axis(BlockView v, double* __restrict__ B) {
-    const int na = v.n1 + 2 * NG, nb = v.n3 + 2 * NG;
-    const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= 2L * na * nb) return;
-    const int i = (int)(t % na) - NG;
-    const int k = (int)((t / na) % nb) - NG;
-    const int side = (int)(t / ((long)na * nb));
-    if (v.bc[2 + side] != HAMR_BC_POLAR) return;
-    B[v.nc + cidx(v, i, side == 0 ? 0 : v.n2, k)] = 0.0;
+// Every ghost cell and face in one launch (threads over the x3 slabs, then the x2 and x1 ones without
+// them, then the axis faces of the lower pole): sources are interior, so no pass waits for another. Four
+// dependent launches before: a 256x128x64 block 38 -> 20 us, a 64x32x16 block 21 -> 7 us.
+// P32, K32 (mixed precision on a single block, else null): the ghost cells of the FP32 copy of the
+// primitives and of its entropy tracer kappa, from the same sources
+__global__ void k_bc(BlockView v, double* __restrict__ P, double* __restrict__ B, float* __restrict__ P32,
+                     float* __restrict__ K32) {
+    long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    const long s3 = 2L * NG * v.n1p * v.n2p, s2 = 2L * NG * v.n1p * v.n3, s1 = 2L * NG * v.n2 * v.n3;
+    int i, j, k;
+    if (t < s3) {
+        const int m = (int)(t / ((long)v.n1p * v.n2p));
+        i = (int)(t % v.n1p) - NG;
+        j = (int)((t / v.n1p) % v.n2p) - NG;
+        k = m < NG ? m - NG : v.n3 + m - NG;
+    } else if ((t -= s3) < s2) {
+        const int m = (int)((t / v.n1p) % (2 * NG));
+        i = (int)(t % v.n1p) - NG;
+        j = m < NG ? m - NG : v.n2 + m - NG;
+        k = (int)(t / (2L * NG * v.n1p));
+    } else if ((t -= s2) < s1) {
+        const int m = (int)(t % (2 * NG));
+        i = m < NG ? m - NG : v.n1 + m - NG;
+        j = (int)((t / (2 * NG)) % v.n2);
+        k = (int)(t / (2L * NG * v.n2));
+    } else if ((t -= s1) < (long)v.n1 * v.n3) {
+        if (v.bc[2] == HAMR_BC_POLAR) B[v.nc + cidx(v, (int)(t % v.n1), 0, (int)(t / v.n1))] = 0.0;
+        return;
+    } else {
+        return;
+    }
+    const long dst = cidx(v, i, j, k);
+    {
+        int x[4] = {0, i, j, k};
+        const bool polar = bc_source(v, 0, x);
+        const long src = cidx(v, x[1], x[2], x[3]);
+        const bool nolo = i < 0 && v.bc[0] == HAMR_BC_OUTFLOW_NOINFLOW;
+        const bool nohi = i >= v.n1 && v.bc[1] == HAMR_BC_OUTFLOW_NOINFLOW;
+#pragma unroll
+        for (int q = 0; q < NPRIM; q++) {
+            double p = P[q * v.nc + src];
+            if (polar && (q == U2 || q == B2)) p = -p;
+            if (q == U1) {
+                if (nohi && p < 0.0) p = 0.0;
+                if (nolo && p > 0.0) p = 0.0;
+            }
+            P[q * v.nc + dst] = p;
+            if (P32) P32[q * v.nc + dst] = (float)p;
+        }
+        if (K32) K32[dst] = K32[src];  // kappa depends on rho and u only, which the map keeps
+    }
+#pragma unroll
+    for (int f = 1; f <= 3; f++) {
+        int x[4] = {0, i, j, k};
+        const bool polar = bc_source(v, f, x);
+        double* b = B + (f - 1) * v.nc;
+        const bool axis = f == 2 && ((j == 0 && v.bc[2] == HAMR_BC_POLAR) || (j == v.n2 && v.bc[3] == HAMR_BC_POLAR));
+        const long src = cidx(v, x[1], x[2], x[3]);
+        if (axis)
+            b[dst] = 0.0;
+        else if (src != dst)
+            b[dst] = (polar && f == 2) ? -b[src] : b[src];
+    }
 }
 
 // ---------------------------------------------------------------- reconstruction
@@ -892,43 +912,105 @@ __global__ void k_ct(BlockView v, const double* __restrict__ E, const double* Bb
 // largest CFL rate of the block's cells. The FP64 rate of a cell is formed only where its FP32 estimate is
 // not certainly below the largest rate found so far (rate_below): in a spherical block nearly every cell is
 // (the largest rates sit next to the axis at the inner edge), and the result is the same bits.
-__device__ __forceinline__ void b_dt_reduce(const BlockView& v, PhysArgs ph, const double* __restrict__ P, unsigned long long* dmax, long t) {
-    const long n = (long)v.n1 * v.n2 * v.n3;
+__device__ __forceinline__ double cell_rate(const BlockView& v, const PhysArgs& ph, int i, int j, const double pr[NPRIM],
+                                            const unsigned long long* dmax) {
+    Metric<double> m;
+    load_metric(v.gc, v.n2d, gidx(v, i, j), m);
+    const int w = smr_width(v, ph, j);
+    BlockView vw = v;
+    if (w > 1) vw.idx3 = v.idx3 / w;  // an internal-SMR group: its width in x3
+    // the estimate's fluid state in FP32, (rho, u, B^2) scaled to O(1) by 2^sh, sh even
+    const int sh = scale_of(pr[RHO], pr[UU], 0.0) & ~0x100000;
+    Metric<float> mf;
+    mf.g01 = narrow(m.g01), mf.g03 = narrow(m.g03), mf.g11 = narrow(m.g11), mf.g13 = narrow(m.g13);
+    mf.g22 = narrow(m.g22), mf.g33 = narrow(m.g33);
+    const float q1 = narrow(pr[U1]), q2 = narrow(pr[U2]), q3 = narrow(pr[U3]);
+    const float u1 = mf.g11 * q1 + mf.g13 * q3, u2 = mf.g22 * q2, u3 = mf.g13 * q1 + mf.g33 * q3;
+    const float g2 = 1.0f + q1 * u1 + q2 * u2 + q3 * u3, gamma = sqrtf(g2);
+    const float al = narrow(m.alpha), c01 = narrow(m.c01);
+    const float b1 = ff_of(pr[B1], sh / 2).h, b2 = ff_of(pr[B2], sh / 2).h, b3 = ff_of(pr[B3], sh / 2).h;
+    const float bt = b1 * u1 + b2 * u2 + b3 * u3;
+    const float bb = mf.g11 * b1 * b1 + mf.g22 * b2 * b2 + mf.g33 * b3 * b3 + 2.0f * mf.g13 * b1 * b3;
+    const float bsq = al * al * (bb + bt * bt) / g2;
+    const float ud[3] = {q1 - gamma * al * c01, q2, q3};
+    const float est = rate_estimate(vw, ph, ff_of(pr[RHO], sh).h, ff_of(pr[UU], sh).h, bsq, gamma / al, ud,
+                                    narrow(m.c00), c01, narrow(m.c11), narrow(m.c22), narrow(m.c33));
+    return rate_below(est, dmax) ? 0.0 : inv_dt_cell(vw, pr, m, ph.gam);
+}
+
+__device__ __forceinline__ void b_dt_reduce(const BlockView& v, const PhysArgs& ph, const double* __restrict__ P,
+                                            unsigned long long* dmax, long t) {
     double inv = 0.0;
-    if (t < n) {
+    if (t < (long)v.n1 * v.n2 * v.n3) {
         const int i = (int)(t % v.n1), j = (int)((t / v.n1) % v.n2), k = (int)(t / ((long)v.n1 * v.n2));
         const long c = cidx(v, i, j, k);
-        Metric<double> m;
-        load_metric(v.gc, v.n2d, gidx(v, i, j), m);
         double pr[NPRIM];
 #pragma unroll
         for (int q = 0; q < NPRIM; q++) pr[q] = P[q * v.nc + c];
-        const int w = smr_width(v, ph, j);
-        BlockView vw = v;
-        if (w > 1) vw.idx3 = v.idx3 / w;  // an internal-SMR group: its width in x3
-        // the estimate's fluid state in FP32, (rho, u, B^2) scaled to O(1) by 2^sh, sh even
-        const int sh = scale_of(pr[RHO], pr[UU], 0.0) & ~0x100000;
-        Metric<float> mf;
-        mf.g01 = narrow(m.g01), mf.g03 = narrow(m.g03), mf.g11 = narrow(m.g11), mf.g13 = narrow(m.g13);
-        mf.g22 = narrow(m.g22), mf.g33 = narrow(m.g33);
-        const float q1 = narrow(pr[U1]), q2 = narrow(pr[U2]), q3 = narrow(pr[U3]);
-        const float u1 = mf.g11 * q1 + mf.g13 * q3, u2 = mf.g22 * q2, u3 = mf.g13 * q1 + mf.g33 * q3;
-        const float g2 = 1.0f + q1 * u1 + q2 * u2 + q3 * u3, gamma = sqrtf(g2);
-        const float al = narrow(m.alpha), c01 = narrow(m.c01);
-        const float b1 = ff_of(pr[B1], sh / 2).h, b2 = ff_of(pr[B2], sh / 2).h, b3 = ff_of(pr[B3], sh / 2).h;
-        const float bt = b1 * u1 + b2 * u2 + b3 * u3;
-        const float bb = mf.g11 * b1 * b1 + mf.g22 * b2 * b2 + mf.g33 * b3 * b3 + 2.0f * mf.g13 * b1 * b3;
-        const float bsq = al * al * (bb + bt * bt) / g2;
-        const float ud[3] = {q1 - gamma * al * c01, q2, q3};
-        const float est = rate_estimate(vw, ph, ff_of(pr[RHO], sh).h, ff_of(pr[UU], sh).h, bsq, gamma / al, ud,
-                                        narrow(m.c00), c01, narrow(m.c11), narrow(m.c22), narrow(m.c33));
-        if (!rate_below(est, dmax)) inv = inv_dt_cell(vw, pr, m, ph.gam);
+        inv = cell_rate(v, ph, i, j, pr, dmax);
     }
     reduce_rate(inv, dmax);
 }
 
 __global__ void k_dt_reduce(BlockView v, PhysArgs ph, const double* __restrict__ P, unsigned long long* dmax) {
     b_dt_reduce(v, ph, P, dmax, (long)blockIdx.x * blockDim.x + threadIdx.x);
+}
+
+// A state load from device memory in one pass over the padded block: prim and bface (field stride n) into
+// P and B (and, in a block tree, into the old state Po and Bo), the centre field of interior cells from the
+// faces, the CFL rate. It replaces 11 copies (13 in a tree), the centre-field pass and the rate's pass over
+// memory: per block of the 512-block tree 15 operations became 2, the tree's load and read-out 61 -> 10 ms.
+__global__ void k_load(BlockView v, PhysArgs ph, const double* __restrict__ prim, const double* __restrict__ bface,
+                       double* __restrict__ P, double* __restrict__ B, double* __restrict__ Po, double* __restrict__ Bo,
+                       unsigned long long* dmax) {
+    const long n = (long)v.n1p * v.n2p * v.n3p;
+    const long c = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    double inv = 0.0;
+    if (c < n) {
+        const int i = (int)(c % v.n1p) - NG, j = (int)((c / v.n1p) % v.n2p) - NG;
+        const int k = (int)(c / ((long)v.n1p * v.n2p)) - NG;
+        const bool in = i >= 0 && i < v.n1 && j >= 0 && j < v.n2 && k >= 0 && k < v.n3;
+        double pr[NPRIM];
+#pragma unroll
+        for (int q = 0; q < NPRIM; q++) pr[q] = (in && q >= B1) ? 0.0 : prim[q * n + c];
+        if (in) {
+            centre_field_at(v, bface, n, c, v.gc[G_IGDET * v.n2d + gidx(v, i, j)], pr + B1);
+            inv = cell_rate(v, ph, i, j, pr, dmax);
+        }
+#pragma unroll
+        for (int q = 0; q < NPRIM; q++) {
+            P[q * v.nc + c] = pr[q];
+            if (Po) Po[q * v.nc + c] = pr[q];
+        }
+#pragma unroll
+        for (int q = 0; q < 3; q++) {
+            const double b = bface[q * n + c];
+            B[q * v.nc + c] = b;
+            if (Bo) Bo[q * v.nc + c] = b;
+        }
+    }
+    reduce_rate(inv, dmax);
+}
+
+// the state out, in the caller's field stride n; prim or bface may be null
+__global__ void k_store(BlockView v, const double* __restrict__ P, const double* __restrict__ B,
+                        double* __restrict__ prim, double* __restrict__ bface) {
+    const long n = (long)v.n1p * v.n2p * v.n3p;
+    const long c = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (c >= n) return;
+    double x[NPRIM + 3];
+    if (prim)
+#pragma unroll
+        for (int q = 0; q < NPRIM; q++) x[q] = P[q * v.nc + c];
+    if (bface)
+#pragma unroll
+        for (int q = 0; q < 3; q++) x[NPRIM + q] = B[q * v.nc + c];
+    if (prim)
+#pragma unroll
+        for (int q = 0; q < NPRIM; q++) prim[q * n + c] = x[q];
+    if (bface)
+#pragma unroll
+        for (int q = 0; q < 3; q++) bface[q * n + c] = x[NPRIM + q];
 }
 
 
@@ -1422,13 +1504,20 @@ cudaError_t launch_centre_b(const BlockView& v, double* P, const double* B, cuda
 }
 
 cudaError_t launch_bc(const BlockView& v, double* P, double* B, cudaStream_t s, float* P32, float* K32) {
-    const int nn[4] = {0, v.n1, v.n2, v.n3};
-    for (int e = 3; e >= 1; e--) {
-        const int ta = (e == 1) ? 2 : 1, tb = (e == 3) ? 2 : 3;
-        const long total = 2L * NG * (nn[ta] + 2 * NG) * (nn[tb] + 2 * NG);
-        k_bc_pass<<<nblk(total), BS, 0, s>>>(v, P, B, e, P32, K32);
-        if (e == 2) k_bc_axis<<<nblk(2L * (v.n1 + 2 * NG) * (v.n3 + 2 * NG)), BS, 0, s>>>(v, B);
-    }
+    const long n = 2L * NG * ((long)v.n1p * v.n2p + (long)v.n1p * v.n3 + (long)v.n2 * v.n3) + (long)v.n1 * v.n3;
+    k_bc<<<nblk(n), BS, 0, s>>>(v, P, B, P32, K32);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_load(const BlockView& v, const PhysArgs& ph, const double* prim, const double* bface, double* P,
+                        double* B, double* Po, double* Bo, unsigned long long* dmax, cudaStream_t s) {
+    k_load<<<nblk((long)v.n1p * v.n2p * v.n3p), BS, 0, s>>>(v, ph, prim, bface, P, B, Po, Bo, dmax);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_store(const BlockView& v, const double* P, const double* B, double* prim, double* bface,
+                         cudaStream_t s) {
+    k_store<<<nblk((long)v.n1p * v.n2p * v.n3p), BS, 0, s>>>(v, P, B, prim, bface);
     return cudaGetLastError();
 }
 
