@@ -323,14 +323,15 @@ __device__ __forceinline__ bool newton_wv_mixed(const C2PScalars& S, double gfac
         const float step = fabsf(dw) + fabsf(dv) * w;
         const float cancel = (fabsf(j11 * j22) + fabsf(j12 * j21)) * fabsf(idet);
         const double Wn = Wd + widen(dw) * ik;
-        const double vn = fmin(fmax(vd + widen(dv), 0.0), C2P_VSQMAX);
-        if (Wn > 0.0 && step < 1e-5f * w && step * cancel < 1e-3f * w) {
+        const double vn = clamp_pos(vd + widen(dv), C2P_VSQMAX);
+        const bool in = is_pos(Wn);
+        if (in && step < 1e-5f * w && step * cancel < 1e-3f * w) {
             it = it32 + 1;
             W = Wn;
             vsq = vn;
             return true;
         }
-        if (Wn > 0.0) {
+        if (in) {
             Wd = Wn;
             vd = vn;
         }
@@ -414,7 +415,7 @@ __device__ __forceinline__ bool energy_result(const C2PScalars& S, double igam, 
     const double sq = omv * rs;
     rho = S.D * sq;
     u = (W * omv - S.D * sq) * igam;
-    return (rho > 0.0) && (u > 0.0);
+    return is_pos(rho) && is_pos(u);
 }
 
 // The inversion in three pieces (invert() below composes them):
@@ -501,9 +502,9 @@ __device__ __forceinline__ void c2p_attempt_p(C2PWork& w, double gam, double p) 
 // one energy-equation attempt from (W, v^2); no-op once an attempt succeeded.
 // The Aitken inversion starts from the pressure of (W, v^2).
 __device__ __forceinline__ void c2p_attempt(C2PWork& w, double gam, double W, double vsq) {
-    if (w.ok || !(W > 0.0)) return;
+    if (w.ok || !is_pos(W)) return;
     const double gfac = w.gfac;
-    vsq = fmin(fmax(vsq, 0.0), C2P_VSQMAX);
+    vsq = clamp_pos(vsq, C2P_VSQMAX);
     if (w.method == HAMR_INV_AITKEN) {
         c2p_attempt_p(w, gam, gfac * (W * (1.0 - vsq) - w.S.D * sqrt(1.0 - vsq)));
         return;

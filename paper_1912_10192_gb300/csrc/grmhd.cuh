@@ -257,6 +257,19 @@ __device__ __forceinline__ T max_i(T a, T b) {
         return ordered_int<T>(FBits<T>::of(a)) >= ordered_int<T>(FBits<T>::of(b)) ? a : b;
 }
 
+// x > 0 and x < 0 on the integer pipe (a double comparison takes the FP64 pipe); false for NaNs
+__device__ __forceinline__ bool is_pos(double x) {
+    const long long b = FBits<double>::of(x);
+    return b > 0 && b <= 0x7FF0000000000000ll;
+}
+__device__ __forceinline__ bool is_neg(double x) { return is_pos(-x); }
+// fmin(fmax(x, 0), hi) for hi > 0 likewise (0 for a NaN)
+__device__ __forceinline__ double clamp_pos(double x, double hi) {
+    const long long b = FBits<double>::of(x);
+    if (!(b > 0 && b <= 0x7FF0000000000000ll)) return 0.0;
+    return b > FBits<double>::of(hi) ? hi : x;
+}
+
 // fastest magnetosonic characteristic speeds along dir (Sec. 2.1): roots of
 // A v^2 - 2 B v + C = 0 with c^2 = vA^2 + cs^2 (1 - vA^2), vA^2 = b^2/(b^2 + w),
 // cs^2 = gam p / w, i.e. c^2 = (b^2 + gam p)/(b^2 + w). The quadratic is taken

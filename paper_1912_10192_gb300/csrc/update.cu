@@ -322,8 +322,10 @@ template <bool COR>
 __global__ void __launch_bounds__(BS) k_update64(BlockView v, PhysArgs ph, HAMR_UPD_PARAMS) {
     b_update64<COR>(v, ph, true, Pf, F1, F2, F3, Bn, Un, Po, status, dscal, fac, dmax, dcnt, tidx());
 }
+// four CTAs per SM (128 registers, a few spilled) without the network: the FP64 pipe waits less between the
+// FP32 stretches (256x128x64 torus, mixed: 0.96 -> 0.92 ms per launch; 384 threads per CTA: 1.09 ms)
 template <bool MLP, typename TS, bool INV64>
-__global__ void __launch_bounds__(BS, 3) k_update(BlockView v, PhysArgs ph, int corrector, HAMR_UPD_PARAMS) {
+__global__ void __launch_bounds__(BS, MLP ? 3 : 4) k_update(BlockView v, PhysArgs ph, int corrector, HAMR_UPD_PARAMS) {
     b_update<MLP, TS, INV64>(v, ph, corrector, Pf, F1, F2, F3, Bn, Un, Po, status, dscal, fac, dmax, dcnt, tidx());
 }
 
@@ -340,7 +342,7 @@ __global__ void __launch_bounds__(BS, 3) kb_update64(const DevBlock* tab, const 
     b_update64<COR>(D.v, ph, false, HAMR_UPD_BLOCK(D, COR));
 }
 template <bool MLP, typename TS, bool INV64>
-__global__ void __launch_bounds__(BS, 3) kb_update(const DevBlock* tab, const int* list, PhysArgs ph, int sigma) {
+__global__ void __launch_bounds__(BS, MLP ? 3 : 4) kb_update(const DevBlock* tab, const int* list, PhysArgs ph, int sigma) {
     const DevBlock& D = tab[list[blockIdx.y]];
     ph.smr_u = D.QR;
     b_update<MLP, TS, INV64>(D.v, ph, sigma ? 2 : 0, HAMR_UPD_BLOCK(D, sigma));
