@@ -120,12 +120,14 @@ __host__ __device__ inline void footprint(const DevBlock& N, const double x[4], 
 struct SrcView {
     const double *Pa, *Pb, *Ba, *Bb;
     double w;
-    __device__ double P(long i) const { return Pb ? Pa[i] + w * (Pb[i] - Pa[i]) : Pa[i]; }
     __device__ double B(long i) const { return Bb ? Ba[i] + w * (Bb[i] - Ba[i]) : Ba[i]; }
 };
 
 // 2^e as a double, built from its bits (-1022 <= e <= 1023): exact, and no work for the FP64 pipe
 __device__ inline double pow2i(int e) { return __hiloint2double((1023 + e) << 20, 0); }
+
+// e / 8 for a small integer: exact in binary32, widened on the integer pipe
+__device__ inline double eighths(int e) { return widen((float)e * 0.125f); }
 
 __device__ inline SrcView source_view(const DevBlock& R, const DevBlock& N, int sigma, int s) {
     SrcView v;
@@ -140,7 +142,7 @@ __device__ inline SrcView source_view(const DevBlock& R, const DevBlock& N, int 
         if (k != 0) {  // else the source's old state itself
             v.Pb = N.P;
             v.Bb = N.B;
-            v.w = (double)k * pow2i(-(N.lat + 1));
+            v.w = widen((float)k * __uint_as_float((unsigned)(127 - (N.lat + 1)) << 23));  // exact, k < 2^24
         }
     } else if (N.lat == R.lat && sigma == 1) {
         v.Pa = N.Ph;
@@ -255,56 +257,80 @@ __device__ inline void ghost_cell_locate(const AmrDomain& A, const DevBlock& R, 
     G.c0 = pidx(N.v, i0[1], i0[2], i0[3]);
 }
 
-// the value of a located ghost cell at stage sigma of substep s into P (or Ph) of R at t
+// Primitives Q0 .. Q0 + GQ - 1 of a located ghost cell at stage sigma of substep s into P (or Ph) of R at t.
+// Bound by the FP64 pipe on large trees (70% busy; 22 instructions per thread, most of them where one lane
+// of a warp prolongs or interpolates in time) and by the latency of the gathers on small ones: the values of
+// all GQ primitives at a source location are asked for together (every decision is the location's, none a
+// primitive's), none is stored before all are formed, and two threads share a ghost cell; offsets, weight and
+// the clamp's comparisons stay off the FP64 pipe. Small box tree: 21.1 -> 9.5 us per launch, 512-block tree
+// 28.0 -> 25.8 ms per period (32.3 with four threads per ghost cell).
+constexpr int GQ = 4;
 __device__ inline void ghost_cell_apply(const AmrDomain& A, const DevBlock& R, const GhostGeo& G, long t, int sigma,
-                                        int s) {
+                                        int s, int Q0) {
     if (G.n < 0) return;
     const DevBlock& N = A.tab[G.n];
     const SrcView S = source_view(R, N, sigma, s);
-    const long sj = N.v.n1p, sk = (long)N.v.n1p * N.v.n2p;
+    const long nc = N.v.nc, sj = N.v.n1p, sk = (long)N.v.n1p * N.v.n2p;
     const long st[4] = {0, 1, sj, sk};
-    const bool one = G.cnt[1] * G.cnt[2] * G.cnt[3] == 1;
-    const double inv = inv_count(G.cnt[1], G.cnt[2], G.cnt[3]);
-    double f[4];  // the prolongation offsets in source cells (multiples of 1/8: exact)
-    for (int d = 1; d <= 3; d++) f[d] = (G.e8[d] == 0) ? 0.0 : (double)G.e8[d] * 0.125;
-    double* out = sigma ? R.Ph : R.P;
-    // source cell c of primitive q, with its MINMOD slopes where prolonged
-    auto cell = [&](int q, long c) {
-        const double q0 = S.P(q * N.v.nc + c);
-        double val = q0;
+    const double* Pa = S.Pa + Q0 * nc;
+    const double* Pb = S.Pb ? S.Pb + Q0 * nc : nullptr;
+    auto load = [&](long c, double x[GQ]) {
+#pragma unroll
+        for (int q = 0; q < GQ; q++) x[q] = Pa[q * nc + c];
+        if (Pb) {
+            double y[GQ];
+#pragma unroll
+            for (int q = 0; q < GQ; q++) y[q] = Pb[q * nc + c];
+#pragma unroll
+            for (int q = 0; q < GQ; q++) x[q] = x[q] + S.w * (y[q] - x[q]);
+        }
+    };
+    // source cell c with its MINMOD slopes where prolonged (offsets in source cells, multiples of 1/8: exact)
+    auto cell = [&](long c, double val[GQ]) {
+        double x[GQ];
+        load(c, x);
+#pragma unroll
+        for (int q = 0; q < GQ; q++) val[q] = x[q];
+#pragma unroll
         for (int d = 1; d <= 3; d++) {
             if (G.e8[d] == 0) continue;
-            const double qm = S.P(q * N.v.nc + c - st[d]);
-            const double qp = S.P(q * N.v.nc + c + st[d]);
-            val += f[d] * minmod_(q0 - qm, qp - q0);
+            const double f = eighths(G.e8[d]);
+            double xm[GQ], xp[GQ];
+            load(c - st[d], xm);
+            load(c + st[d], xp);
+#pragma unroll
+            for (int q = 0; q < GQ; q++) val[q] += f * minmod_(x[q] - xm[q], xp[q] - x[q]);
         }
-        return val;
     };
-    // every primitive is formed before any is stored, so that the gathers of all eight are in
-    // flight together (a store between them could alias the next source and would serialise them)
-    double ov[NPRIM];
-    if (one) {  // a copy or a prolongation: one source cell, no sum
-#pragma unroll
-        for (int q = 0; q < NPRIM; q++) ov[q] = cell(q, G.c0);
+    double ov[GQ];
+    if (G.cnt[1] * G.cnt[2] * G.cnt[3] == 1) {  // a copy or a prolongation: one source cell, no sum
+        cell(G.c0, ov);
     } else {  // the mean of the covered finer cells
+        const double inv = inv_count(G.cnt[1], G.cnt[2], G.cnt[3]);
+        double sum[GQ];
 #pragma unroll
-        for (int q = 0; q < NPRIM; q++) {
-            double sum = 0.0;
-            for (int c3 = 0; c3 < G.cnt[3]; c3++)
-                for (int c2 = 0; c2 < G.cnt[2]; c2++)
-                    for (int c1 = 0; c1 < G.cnt[1]; c1++) sum += cell(q, G.c0 + c1 + c2 * sj + c3 * sk);
-            ov[q] = sum * inv;
-        }
+        for (int q = 0; q < GQ; q++) sum[q] = 0.0;
+        for (int c3 = 0; c3 < G.cnt[3]; c3++)
+            for (int c2 = 0; c2 < G.cnt[2]; c2++)
+                for (int c1 = 0; c1 < G.cnt[1]; c1++) {
+                    double v[GQ];
+                    cell(G.c0 + c1 + c2 * sj + c3 * sk, v);
+#pragma unroll
+                    for (int q = 0; q < GQ; q++) sum[q] += v[q];
+                }
+#pragma unroll
+        for (int q = 0; q < GQ; q++) ov[q] = sum[q] * inv;
     }
+    double* out = (sigma ? R.Ph : R.P) + t;
 #pragma unroll
-    for (int q = 0; q < NPRIM; q++) {
+    for (int q = 0; q < GQ; q++) {
         double o = ov[q];
-        if (G.neg && (q == U2 || q == B2)) o = -o;
-        if (q == U1) {
-            if (G.clamp > 0 && o < 0.0) o = 0.0;
-            if (G.clamp < 0 && o > 0.0) o = 0.0;
+        if (G.neg && (Q0 + q == U2 || Q0 + q == B2)) o = -o;
+        if (Q0 + q == U1) {
+            if (G.clamp > 0 && is_neg(o)) o = 0.0;
+            if (G.clamp < 0 && is_pos(o)) o = 0.0;
         }
-        out[q * R.v.nc + t] = o;
+        out[(Q0 + q) * R.v.nc] = o;
     }
 }
 
@@ -355,7 +381,7 @@ __device__ inline void ghost_face_apply(const AmrDomain& A, const DevBlock& R, c
     const long sj = N.v.n1p, sk = (long)N.v.n1p * N.v.n2p;
     const long st = (fd == 1) ? 1 : ((fd == 2) ? sj : sk);
     const int e8 = G.e8[fd];
-    const double fr = (e8 == 0) ? 0.0 : (double)e8 * 0.125;
+    const double fr = eighths(e8);
     const bool one = G.cnt[1] * G.cnt[2] * G.cnt[3] == 1;
     const double inv = inv_count(G.cnt[1], G.cnt[2], G.cnt[3]);
     auto face = [&](long c) {  // source face c, linear toward the next where between two
@@ -414,7 +440,7 @@ __global__ void k_ghost_cells(AmrDomain A, const int* list, int sigma, int s) {
     if (!ghost_cell_at(R.v, t, i, j, k)) return;
     GhostGeo G;
     ghost_cell_locate(A, R, i, j, k, G);
-    ghost_cell_apply(A, R, G, t, sigma, s);
+    for (int q0 = 0; q0 < NPRIM; q0 += GQ) ghost_cell_apply(A, R, G, t, sigma, s, q0);
 }
 
 __global__ void k_ghost_faces(AmrDomain A, const int* list, int sigma, int s) {
@@ -466,7 +492,7 @@ __global__ void k_ghost_cells_mapped(AmrDomain A, const int* list, int sigma, in
     const GhostLoc L = loc[R.gofs_cell + g];
     GhostGeo G;
     unpack_loc(L, G);
-    ghost_cell_apply(A, R, G, L.t, sigma, s);
+    ghost_cell_apply(A, R, G, L.t, sigma, s, GQ * (int)blockIdx.z);
 }
 
 __global__ void k_ghost_faces_mapped(AmrDomain A, const int* list, int sigma, int s, const GhostLoc* loc) {
@@ -1080,9 +1106,9 @@ struct AmrImpl {
     std::vector<std::vector<int>> lev;  // blocks of each level
     std::vector<int*> dlev;             // device copies
     int* dall = nullptr;                // all blocks
-    long mw_pad = 0, mw_recon = 0, mw_flux[4] = {0, 0, 0, 0}, mw_edge = 0, mw_cell = 0;
+    long mw_pad = 0, mw_flux[4] = {0, 0, 0, 0}, mw_edge = 0, mw_cell = 0;
     std::vector<long> lmw_pad, lmw_edge, lmw_cell, lmw_ext;
-    std::vector<std::vector<long>> lmw_flux, lmw_recon;
+    std::vector<std::vector<long>> lmw_flux;
     // synchronisation
     SyncDev fs{}, es{};
     std::vector<int> fs_beg, fs_end, es_beg, es_end;
@@ -1659,7 +1685,6 @@ int amr_create(AmrImpl** out, const hamr_grid_desc& d, const std::vector<BlockVi
     }
     for (int L = 0; L <= M->Lmax; L++) M->dlev_smr.push_back(M->dev(M->lev_smr[L]));
     M->lmw_pad.assign(M->Lmax + 1, 0);
-    M->lmw_recon.assign(M->Lmax + 1, std::vector<long>(4, 0));
     M->lmw_edge.assign(M->Lmax + 1, 0);
     M->lmw_cell.assign(M->Lmax + 1, 0);
     M->lmw_ext.assign(M->Lmax + 1, 0);
@@ -1671,9 +1696,6 @@ int amr_create(AmrImpl** out, const hamr_grid_desc& d, const std::vector<BlockVi
         const long edg = (long)(v.n1 + 1) * (v.n2 + 1) * (v.n3 + 1);
         const long cel = (long)v.n1 * v.n2 * v.n3;
         M->lmw_pad[L] = std::max(M->lmw_pad[L], pad);
-        for (int dir = 1; dir <= 3; dir++)
-            M->lmw_recon[L][dir] =
-                std::max(M->lmw_recon[L][dir], recon_threads(v, dir, ph.mixed, ph.recon_seg, ph.recon_x1_sweep));
         M->lmw_edge[L] = std::max(M->lmw_edge[L], edg);
         M->lmw_cell[L] = std::max(M->lmw_cell[L], cel);
         M->lmw_ext[L] = std::max(M->lmw_ext[L], (long)(v.n1 + 2) * (v.n2 + 2) * (v.n3 + 2));
@@ -1732,6 +1754,15 @@ namespace {
         if (e_ != cudaSuccess) return set_error(HAMR_ECUDA, "%s failed: %s", #call, cudaGetErrorString(e_)); \
     } while (0)
 
+// the edge values of a level's blocks
+cudaError_t recon_level(const AmrImpl& M, int L, const PhysArgs& ph, int dir, int sigma, cudaStream_t cs) {
+    const int nl = (int)M.lev[L].size();
+    const int m = ph.mixed ? recon_cells(M.lmw_cell[L] * nl, dir) : 0;
+    long mw = 0;
+    for (int b : M.lev[L]) mw = std::max(mw, recon_threads(M.H.b[b].v, dir, m, ph.recon_seg, ph.recon_x1_sweep));
+    return launch_recon_batch(M.dtab, M.dlev[L], nl, mw, m, ph, dir, sigma, cs);
+}
+
 int group_step(AmrImpl& M, int L, int s, cudaStream_t cs) {
     const int nl = (int)M.lev[L].size();
     const int* list = M.dlev[L];
@@ -1741,7 +1772,7 @@ int group_step(AmrImpl& M, int L, int s, cudaStream_t cs) {
     for (int sigma = 0; sigma < 2; sigma++) {
         if (M.use_maps) {
             if (M.lmw_gc[L])
-                k_ghost_cells_mapped<<<dim3(nb_(M.lmw_gc[L]), nl), BSA, 0, cs>>>(M.H.A, list, sigma, s, M.gloc_cell);
+                k_ghost_cells_mapped<<<dim3(nb_(M.lmw_gc[L]), nl, NPRIM / GQ), BSA, 0, cs>>>(M.H.A, list, sigma, s, M.gloc_cell);
             if (M.lmw_gf[L])
                 k_ghost_faces_mapped<<<dim3(nb_(M.lmw_gf[L]), nl), BSA, 0, cs>>>(M.H.A, list, sigma, s, M.gloc_face);
         } else {
@@ -1753,7 +1784,7 @@ int group_step(AmrImpl& M, int L, int s, cudaStream_t cs) {
         AM_TRY(launch_kappa_batch(tab, list, nl, M.lmw_pad[L], ph, sigma, cs));
         for (int dir = 1; dir <= 3; dir++) {
             if (ph.flatten) AM_TRY(launch_flatten_batch(tab, list, nl, M.lmw_ext[L], ph, dir, sigma, cs));
-            AM_TRY(launch_recon_batch(tab, list, nl, M.lmw_recon[L][dir], ph, dir, sigma, cs));
+            AM_TRY(recon_level(M, L, ph, dir, sigma, cs));
             AM_TRY(launch_flux_batch(tab, list, nl, M.lmw_flux[L][dir], ph, dir, sigma, cs));
         }
         const int fb = M.fs_beg[L], fe = M.fs_end[L];
@@ -1866,13 +1897,6 @@ int amr_period(AmrImpl* M, cudaStream_t s, int nperiods, bool use_graph) {
 
 int amr_set_phys(AmrImpl* M, const PhysArgs& ph) {
     M->ph = ph;  // the captured period bakes the launch arguments: capture again
-    for (int L = 0; L <= M->Lmax; L++)
-        for (int dir = 1; dir <= 3; dir++) {
-            long mw = 0;
-            for (int b : M->lev[L])
-                mw = std::max(mw, recon_threads(M->H.b[b].v, dir, ph.mixed, ph.recon_seg, ph.recon_x1_sweep));
-            M->lmw_recon[L][dir] = mw;
-        }
     if (M->exec) cudaGraphExecDestroy(M->exec);
     if (M->graph) cudaGraphDestroy(M->graph);
     M->exec = nullptr;
@@ -1895,13 +1919,6 @@ int amr_time_group(AmrImpl* M, const PhysArgs& ph, int which, cudaStream_t cs, f
         const int nl = (int)M->lev[L].size();
         if (!nl) continue;
         const int* list = M->dlev[L];
-        long mwr[4];
-        for (int dir = 1; dir <= 3; dir++) {
-            mwr[dir] = 0;
-            for (int bb : M->lev[L])
-                mwr[dir] = std::max(mwr[dir], recon_threads(M->H.b[bb].v, dir, ph.mixed, ph.recon_seg,
-                                                            ph.recon_x1_sweep));
-        }
         auto timed = [&](auto launch) {
             cudaEventRecord(a, cs);
             cudaError_t e = launch();
@@ -1931,7 +1948,7 @@ int amr_time_group(AmrImpl* M, const PhysArgs& ph, int which, cudaStream_t cs, f
             auto rec = [&]() {
                 cudaError_t e = ph.flatten ? launch_flatten_batch(tab, list, nl, M->lmw_ext[L], ph, dir, 0, cs)
                                            : cudaSuccess;
-                return e == cudaSuccess ? launch_recon_batch(tab, list, nl, mwr[dir], ph, dir, 0, cs) : e;
+                return e == cudaSuccess ? recon_level(*M, L, ph, dir, 0, cs) : e;
             };
             auto flx = [&]() { return launch_flux_batch(tab, list, nl, M->lmw_flux[L][dir], ph, dir, 0, cs); };
             if (which == 0) {
@@ -1959,7 +1976,7 @@ int amr_fill(AmrImpl* M, cudaStream_t s) {
         if (!nl) continue;
         if (M->use_maps) {
             if (M->lmw_gc[L])
-                k_ghost_cells_mapped<<<dim3(nb_(M->lmw_gc[L]), nl), BSA, 0, s>>>(M->H.A, M->dlev[L], 0, 0, M->gloc_cell);
+                k_ghost_cells_mapped<<<dim3(nb_(M->lmw_gc[L]), nl, NPRIM / GQ), BSA, 0, s>>>(M->H.A, M->dlev[L], 0, 0, M->gloc_cell);
             if (M->lmw_gf[L])
                 k_ghost_faces_mapped<<<dim3(nb_(M->lmw_gf[L]), nl), BSA, 0, s>>>(M->H.A, M->dlev[L], 0, 0, M->gloc_face);
         } else {

@@ -105,13 +105,18 @@ __host__ __device__ inline int smr_rows(const BlockView& v, const PhysArgs& ph) 
 
 // threads of one reconstruction launch (FP64): rows along x1 in warps of 32
 // lanes that produce RECON_TILE cells each; pencils along x2 or x3 of
-// RECON_SEG cells per thread; 7 variables each. FP32: one thread per cell.
+// RECON_SEG cells per thread; 7 variables each. FP32 (m > 0): m cells per
+// thread along dir, all variables.
 constexpr int RECON_TILE = 28;
 constexpr int RECON_SEG = 16;  // default sweep length
 constexpr int RECON_X1_SWEEP = 1;  // default form of the x1 edge values
-__host__ __device__ inline long recon_threads(const BlockView& v, int dir, int fp32, int seg, int x1_sweep = 0) {
+// FP32: cells per thread along dir for a launch over this many cells (4, along x1 2, where that leaves 8 warps
+// or so per scheduler of the 152 SMs, b_recon_cells)
+inline int recon_cells(long cells, int dir) { return cells < 152L * 4 * 8 * 32 * 4 ? 1 : (dir == 1 ? 2 : 4); }
+__host__ __device__ inline long recon_threads(const BlockView& v, int dir, int m, int seg, int x1_sweep = 0) {
     const long n1 = v.n1 + 2, n2 = v.n2 + 2, n3 = v.n3 + 2;
-    if (fp32) return n1 * n2 * n3;  // one thread per cell
+    if (m > 0)
+        return dir == 1 ? (n1 + m - 1) / m * n2 * n3 : (dir == 2 ? n1 * ((n2 + m - 1) / m) * n3 : n1 * n2 * ((n3 + m - 1) / m));
     // 8 variables: the 7 primitives other than B^dir and the entropy tracer
     if (dir == 1 && !x1_sweep) return ((n1 + RECON_TILE - 1) / RECON_TILE) * 32 * n2 * n3 * 8;
     if (dir == 1) return n2 * n3 * ((n1 + seg - 1) / seg) * 8;
@@ -281,8 +286,9 @@ cudaError_t launch_to_f32_batch(const DevBlock* tab, const int* list, int nlist,
 // kappa of each listed block into field 0 of its EMF array (maxwork: largest padded cell count)
 cudaError_t launch_kappa_batch(const DevBlock* tab, const int* list, int nlist, long maxwork, const PhysArgs& ph,
                                int sigma, cudaStream_t s);
-cudaError_t launch_recon_batch(const DevBlock* tab, const int* list, int nlist, long maxwork, const PhysArgs& ph,
-                               int dir, int sigma, cudaStream_t s);
+// m: cells per thread in FP32 (recon_cells; maxwork is counted with it)
+cudaError_t launch_recon_batch(const DevBlock* tab, const int* list, int nlist, long maxwork, int m,
+                               const PhysArgs& ph, int dir, int sigma, cudaStream_t s);
 // maxcells: largest (n1 + 2)(n2 + 2)(n3 + 2) of the listed blocks
 cudaError_t launch_flatten_batch(const DevBlock* tab, const int* list, int nlist, long maxcells, const PhysArgs& ph,
                                  int dir, int sigma, cudaStream_t s);

@@ -342,48 +342,69 @@ __device__ __forceinline__ void b_recon_sweep(const BlockView& v, PhysArgs ph, c
     }
 }
 
-// one thread per cell (FP32: the slope and interface arithmetic is cheap next to
-// the loads, and a thread per cell keeps more loads in flight than a sweep)
-template <int DIR, typename T>
-__device__ __forceinline__ void b_recon_cell(const BlockView& v, PhysArgs ph, const T* __restrict__ P,
-                                             const T* __restrict__ K, const T* __restrict__ Fl,
-                                             T* __restrict__ QL, T* __restrict__ QR, long t) {
-    const int e1 = v.n1 + 2, e2 = v.n2 + 2, e3 = v.n3 + 2;
+// FP32: M cells per thread along dir, their M + 4 values of a variable loaded together (a sweep that loads
+// cell by cell is latency-bound), every slope and interface value formed once for them. Bound by
+// instruction issue (comparisons and selects run at half rate) on large launches: with M = 4 a cell takes
+// 1.5 slopes and 1.25 interface values instead of 3 and 2 (256x128x64 torus, x2 / x3: 91 / 83 -> 58 / 73 us;
+// x1 with M = 2: 61 -> 60). On small launches the threads are what is missing: M = 1 (53x37x22:
+// 5.8 us per direction, 9 with M = 4).
+template <int DIR, int M, typename T>
+__device__ __forceinline__ void b_recon_cells(const BlockView& v, PhysArgs ph, const T* __restrict__ P,
+                                              const T* __restrict__ K, const T* __restrict__ Fl,
+                                              T* __restrict__ QL, T* __restrict__ QR, long t) {
+    const int nd = (DIR == 1) ? v.n1 : ((DIR == 2) ? v.n2 : v.n3);
+    const int ng = (nd + 2 + M - 1) / M;  // groups of cells -1 .. nd
+    const int e1 = (DIR == 1) ? ng : v.n1 + 2, e2 = (DIR == 2) ? ng : v.n2 + 2, e3 = (DIR == 3) ? ng : v.n3 + 2;
     if (t >= (long)e1 * e2 * e3) return;
-    const int i = (int)(t % e1) - 1, j = (int)((t / e1) % e2) - 1, k = (int)(t / ((long)e1 * e2)) - 1;
-    const long c = cidx(v, i, j, k);
+    const int x1 = (int)(t % e1), x2 = (int)((t / e1) % e2), x3 = (int)(t / ((long)e1 * e2));
+    const int a0 = M * ((DIR == 1) ? x1 : ((DIR == 2) ? x2 : x3)) - 1;  // the first cell along dir
+    const long c = cidx(v, (DIR == 1) ? a0 : x1 - 1, (DIR == 2) ? a0 : x2 - 1, (DIR == 3) ? a0 : x3 - 1);
     const long st = (DIR == 1) ? 1 : ((DIR == 2) ? (long)v.n1p : (long)v.n1p * v.n2p);
-#pragma unroll
+#pragma unroll (M == 1 ? 8 : 2)
     for (int n = 0; n < 8; n++) {
-        const int q = recon_dst<DIR>(n);
+        const long q = (long)recon_dst<DIR>(n) * v.nc + c;
         const T* p = recon_src<DIR>(v, n, P, K) + c;
-        T l, r;
+        T x[M + 4];
+#pragma unroll
+        for (int m = 0; m < M + 4; m++)  // the last group stays in the block
+            x[m] = p[(M == 1 ? m - 2 : min(m - 2, nd + 2 - a0)) * st];
         if (ph.recon == HAMR_RECON_PPM) {
-            const T qmm = p[-2 * st], qm = p[-st], qc = p[0], qp = p[st], qpp = p[2 * st];
-            const T dmm = qm - qmm, dm = qc - qm, dp = qp - qc, dpp = qpp - qp;
-            const T sm = mc_slope_d(dmm, dm, qc - qmm), sc = mc_slope_d(dm, dp, qp - qm),
-                    sp = mc_slope_d(dp, dpp, qpp - qc);
-            l = ppm_face_d(qm, dm, sm, sc);
-            r = ppm_face_d(qc, dp, sc, sp);
-            if (ph.flatten) flatten_edges(Fl[c], qc, l, r);
-            ppm_limit(qc, l, r);
+            T d[M + 3], sl[M + 2], f[M + 1];
+#pragma unroll
+            for (int m = 0; m < M + 3; m++) d[m] = x[m + 1] - x[m];
+#pragma unroll
+            for (int m = 0; m < M + 2; m++) sl[m] = mc_slope_d(d[m], d[m + 1], x[m + 2] - x[m]);
+#pragma unroll
+            for (int m = 0; m < M + 1; m++) f[m] = ppm_face_d(x[m + 1], d[m + 1], sl[m], sl[m + 1]);
+#pragma unroll
+            for (int m = 0; m < M; m++) {
+                if (a0 + m > nd) break;
+                T l = f[m], r = f[m + 1];
+                if (ph.flatten) flatten_edges(Fl[c + m * st], x[m + 2], l, r);
+                ppm_limit(x[m + 2], l, r);
+                QL[q + m * st] = l;
+                QR[q + m * st] = r;
+            }
         } else {
-            const T dq = limited_slope(ph.recon, p[-st], p[0], p[st]);
-            l = p[0] - T(0.5) * dq;
-            r = p[0] + T(0.5) * dq;
+#pragma unroll
+            for (int m = 0; m < M; m++) {
+                if (a0 + m > nd) break;
+                const T dq = limited_slope(ph.recon, x[m + 1], x[m + 2], x[m + 3]);
+                QL[q + m * st] = x[m + 2] - T(0.5) * dq;
+                QR[q + m * st] = x[m + 2] + T(0.5) * dq;
+            }
         }
-        QL[q * v.nc + c] = l;
-        QR[q * v.nc + c] = r;
     }
 }
 
-// FP64: the non-redundant row and pencil forms; FP32: one thread per cell
-template <int DIR, typename T>
+// FP64: the non-redundant row and pencil forms; FP32: a few cells per thread
+// M: cells per thread in FP32 (0: FP64)
+template <int DIR, typename T, int M>
 __device__ __forceinline__ void b_recon(const BlockView& v, PhysArgs ph, const T* __restrict__ P,
                                         const T* __restrict__ K, const T* __restrict__ Fl, T* __restrict__ QL,
                                         T* __restrict__ QR, long t) {
-    if constexpr (!std::is_same<T, double>::value)
-        b_recon_cell<DIR>(v, ph, P, K, Fl, QL, QR, t);
+    if constexpr (M > 0)
+        b_recon_cells<DIR, M>(v, ph, P, K, Fl, QL, QR, t);
     else if constexpr (DIR == 1) {
         if (ph.recon_x1_sweep)
             b_recon_sweep<1>(v, ph, P, K, Fl, QL, QR, t);
@@ -394,10 +415,10 @@ __device__ __forceinline__ void b_recon(const BlockView& v, PhysArgs ph, const T
     }
 }
 
-template <int DIR, typename T>
+template <int DIR, typename T, int M>
 __global__ void k_recon(BlockView v, PhysArgs ph, const T* __restrict__ P, const T* __restrict__ K,
                         const T* __restrict__ Fl, T* __restrict__ QL, T* __restrict__ QR) {
-    b_recon<DIR, T>(v, ph, P, K, Fl, QL, QR, (long)blockIdx.x * blockDim.x + threadIdx.x);
+    b_recon<DIR, T, M>(v, ph, P, K, Fl, QL, QR, (long)blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 // FP32 copy of the 8 primitive fields over the whole padded block (mixed precision)
@@ -1031,14 +1052,14 @@ __global__ void k_dt_select(double cour, double user_dt, double* dscal, unsigned
 
 // kappa goes to field 0 of the EMF array (free until the EMFs), the flattening
 // coefficients of dir to field 0 of the dir-flux array
-template <int DIR, typename T>
+template <int DIR, typename T, int M>
 __global__ void kb_recon(const DevBlock* tab, const int* list, PhysArgs ph, int sigma) {
     const DevBlock& D = tab[list[blockIdx.y]];
     const double* Fl = (DIR == 1) ? D.F1 : ((DIR == 2) ? D.F2 : D.F3);
     if constexpr (std::is_same<T, double>::value)
-        b_recon<DIR, T>(D.v, ph, sigma ? D.Ph : D.P, D.E, Fl, D.QL, D.QR, tidx());
+        b_recon<DIR, T, M>(D.v, ph, sigma ? D.Ph : D.P, D.E, Fl, D.QL, D.QR, tidx());
     else  // the FP32 copy holds the stage's state
-        b_recon<DIR, T>(D.v, ph, D.P32, reinterpret_cast<const float*>(D.E), reinterpret_cast<const float*>(Fl),
+        b_recon<DIR, T, M>(D.v, ph, D.P32, reinterpret_cast<const float*>(D.E), reinterpret_cast<const float*>(Fl),
                         reinterpret_cast<float*>(D.QL), reinterpret_cast<float*>(D.QR), tidx());
 }
 
@@ -1550,7 +1571,8 @@ cudaError_t launch_kappa(const BlockView& v, const PhysArgs& ph, const double* P
 
 cudaError_t launch_recon(const BlockView& v, const PhysArgs& ph, int dir, const double* P, const float* P32,
                          const double* K, const double* Fl, double* QL, double* QR, cudaStream_t s) {
-    const long n = recon_threads(v, dir, ph.mixed, ph.recon_seg, ph.recon_x1_sweep);
+    const int m = recon_cells((long)v.n1 * v.n2 * v.n3, dir);
+    const long n = recon_threads(v, dir, ph.mixed ? m : 0, ph.recon_seg, ph.recon_x1_sweep);
     const unsigned nb = nblk(n, ph.bs_recon);
     const int bs = ph.bs_recon;
     if (ph.mixed) {
@@ -1558,13 +1580,13 @@ cudaError_t launch_recon(const BlockView& v, const PhysArgs& ph, int dir, const 
         const float* F32 = reinterpret_cast<const float*>(Fl);
         float* L = reinterpret_cast<float*>(QL);
         float* R = reinterpret_cast<float*>(QR);
-        if (dir == 1) k_recon<1, float><<<nb, bs, 0, s>>>(v, ph, P32, K32, F32, L, R);
-        if (dir == 2) k_recon<2, float><<<nb, bs, 0, s>>>(v, ph, P32, K32, F32, L, R);
-        if (dir == 3) k_recon<3, float><<<nb, bs, 0, s>>>(v, ph, P32, K32, F32, L, R);
+        if (dir == 1) (m == 1 ? k_recon<1, float, 1> : k_recon<1, float, 2>)<<<nb, bs, 0, s>>>(v, ph, P32, K32, F32, L, R);
+        if (dir == 2) (m == 1 ? k_recon<2, float, 1> : k_recon<2, float, 4>)<<<nb, bs, 0, s>>>(v, ph, P32, K32, F32, L, R);
+        if (dir == 3) (m == 1 ? k_recon<3, float, 1> : k_recon<3, float, 4>)<<<nb, bs, 0, s>>>(v, ph, P32, K32, F32, L, R);
     } else {
-        if (dir == 1) k_recon<1, double><<<nb, bs, 0, s>>>(v, ph, P, K, Fl, QL, QR);
-        if (dir == 2) k_recon<2, double><<<nb, bs, 0, s>>>(v, ph, P, K, Fl, QL, QR);
-        if (dir == 3) k_recon<3, double><<<nb, bs, 0, s>>>(v, ph, P, K, Fl, QL, QR);
+        if (dir == 1) k_recon<1, double, 0><<<nb, bs, 0, s>>>(v, ph, P, K, Fl, QL, QR);
+        if (dir == 2) k_recon<2, double, 0><<<nb, bs, 0, s>>>(v, ph, P, K, Fl, QL, QR);
+        if (dir == 3) k_recon<3, double, 0><<<nb, bs, 0, s>>>(v, ph, P, K, Fl, QL, QR);
     }
     return cudaGetLastError();
 }
@@ -1629,19 +1651,19 @@ cudaError_t launch_dt_select(const PhysArgs& ph, double user_dt, double* dscal, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_recon_batch(const DevBlock* tab, const int* list, int nlist, long maxwork, const PhysArgs& ph,
-                               int dir, int sigma, cudaStream_t s) {
+cudaError_t launch_recon_batch(const DevBlock* tab, const int* list, int nlist, long maxwork, int m,
+                               const PhysArgs& ph, int dir, int sigma, cudaStream_t s) {
     if (nlist <= 0) return cudaSuccess;
     const int bs = ph.bs_recon;
     const dim3 g = bgrid(maxwork, nlist, bs);
     if (ph.mixed) {
-        if (dir == 1) kb_recon<1, float><<<g, bs, 0, s>>>(tab, list, ph, sigma);
-        if (dir == 2) kb_recon<2, float><<<g, bs, 0, s>>>(tab, list, ph, sigma);
-        if (dir == 3) kb_recon<3, float><<<g, bs, 0, s>>>(tab, list, ph, sigma);
+        if (dir == 1) (m == 1 ? kb_recon<1, float, 1> : kb_recon<1, float, 2>)<<<g, bs, 0, s>>>(tab, list, ph, sigma);
+        if (dir == 2) (m == 1 ? kb_recon<2, float, 1> : kb_recon<2, float, 4>)<<<g, bs, 0, s>>>(tab, list, ph, sigma);
+        if (dir == 3) (m == 1 ? kb_recon<3, float, 1> : kb_recon<3, float, 4>)<<<g, bs, 0, s>>>(tab, list, ph, sigma);
     } else {
-        if (dir == 1) kb_recon<1, double><<<g, bs, 0, s>>>(tab, list, ph, sigma);
-        if (dir == 2) kb_recon<2, double><<<g, bs, 0, s>>>(tab, list, ph, sigma);
-        if (dir == 3) kb_recon<3, double><<<g, bs, 0, s>>>(tab, list, ph, sigma);
+        if (dir == 1) kb_recon<1, double, 0><<<g, bs, 0, s>>>(tab, list, ph, sigma);
+        if (dir == 2) kb_recon<2, double, 0><<<g, bs, 0, s>>>(tab, list, ph, sigma);
+        if (dir == 3) kb_recon<3, double, 0><<<g, bs, 0, s>>>(tab, list, ph, sigma);
     }
     return cudaGetLastError();
 }
