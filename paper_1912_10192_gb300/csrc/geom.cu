@@ -38,12 +38,73 @@ __device__ void store_metric(double* __restrict__ tab, long stride, long q, cons
     tab[G_IGDET * stride + q] = pole ? 0.0 : 1.0 / M.gdet;
 }
 
-// Sixteen threads per (i, j) point. The point's metric is wanted at eleven places (the centre, four around
-// it in x1 and four in x2 for the derivatives, the two faces), each a chain of FP64 transcendental
-// functions: one place per thread, the covariant entries shared through shared memory, then the Christoffel
-// symbols spread over the threads. Bound by that chain's latency: the tables of a 24x12x8 block, which the
-// no-allocation step forms on every call, took about 90 us more with a thread per point; now 22 us.
-constexpr int GEO_T = 16, GEO_P = 8;  // threads per point, points per CTA
+// One thread per (i, j) point: the least work, for planes that fill the chip with it.
+__global__ void k_geometry_points(GeomArgs A) {
+    const long n2d = A.table_stride;
+    const long q = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= (long)A.n1p * A.n2p) return;
+    const int i = (int)(q % A.n1p) - NG;
+    const int j = (int)(q / A.n1p) - NG;
+    const double x1c = A.x1min + (i + 0.5) * A.dx1, x2c = A.x2min + (j + 0.5) * A.dx2;
+    const double x1f = A.x1min + i * A.dx1, x2f = A.x2min + j * A.dx2;
+    FullMetric M;
+    metric_at(A.metric, A.a, x1c, x2c, M);
+    store_metric(A.centre, n2d, q, M, false);
+    // Christoffel symbols at the centre
+    double dg[3][4][4];  // d/dx1, d/dx2 (index 1, 2); index 0 unused
+    for (int m = 0; m < 4; m++)
+        for (int n = 0; n < 4; n++) dg[0][m][n] = dg[1][m][n] = dg[2][m][n] = 0.0;
+    if (A.metric != HAMR_METRIC_MINKOWSKI) {
+        for (int s = 1; s <= 2; s++) {
+            const double e1 = (s == 1) ? CONN_H : 0.0, e2 = (s == 2) ? CONN_H : 0.0;
+            FullMetric p2, p1, m1, m2;
+            metric_at(A.metric, A.a, x1c + 2.0 * e1, x2c + 2.0 * e2, p2);
+            metric_at(A.metric, A.a, x1c + e1, x2c + e2, p1);
+            metric_at(A.metric, A.a, x1c - e1, x2c - e2, m1);
+            metric_at(A.metric, A.a, x1c - 2.0 * e1, x2c - 2.0 * e2, m2);
+            for (int m = 0; m < 4; m++)
+                for (int n = 0; n < 4; n++)
+                    dg[s][m][n] = (8.0 * (p1.g[m][n] - m1.g[m][n]) - (p2.g[m][n] - m2.g[m][n])) / (12.0 * CONN_H);
+        }
+    }
+    // Gamma^l_{mn} = 1/2 g^{lk} (d_m g_{kn} + d_n g_{km} - d_k g_{mn})
+    for (int l = 0; l < 4; l++)
+        for (int m = 0; m < 4; m++)
+            for (int n = m; n < 4; n++) {
+                double s = 0.0;
+                for (int k = 0; k < 4; k++) {
+                    const double dm = (m == 1 || m == 2) ? dg[m][k][n] : 0.0;
+                    const double dn = (n == 1 || n == 2) ? dg[n][k][m] : 0.0;
+                    const double dk = (k == 1 || k == 2) ? dg[k][m][n] : 0.0;
+                    s += M.gi[l][k] * (dm + dn - dk);
+                }
+                A.centre[(C_CONN + l * 10 + sym(m, n)) * n2d + q] = 0.5 * s;
+            }
+    {
+        const int pm[7] = {0, 0, 0, 1, 1, 2, 3}, pn[7] = {0, 1, 3, 1, 3, 2, 3};
+        for (int s = 1; s <= 2; s++)
+            for (int p = 0; p < 7; p++)
+                A.centre[(C_DG + (s - 1) * 7 + p) * n2d + q] = (pm[p] == pn[p] ? 0.5 : 1.0) * dg[s][pm[p]][pn[p]];
+    }
+    const double r = (A.metric != HAMR_METRIC_MINKOWSKI) ? exp(x1c) : 1.0;
+    A.centre[C_RHOFLR * n2d + q] = 1.0e-7 / (r * r);
+    A.centre[C_UFLR * n2d + q] = 1.0e-9 * pow(r, -10.0 / 3.0);
+
+    metric_at(A.metric, A.a, x1f, x2c, M);
+    store_metric(A.face1, n2d, q, M, false);
+    metric_at(A.metric, A.a, x1c, x2f, M);
+    const bool pole = (A.pole_lo && j == 0) || (A.pole_hi && j == A.n2);
+    store_metric(A.face2, n2d, q, M, pole);
+}
+
+// Twelve threads per (i, j) point, for smaller planes. The point's metric is wanted at eleven places (the
+// centre, four around it in x1 and four in x2 for the derivatives, the two faces), each a chain of FP64
+// transcendental functions: one place per thread, the covariant entries shared through shared memory, then
+// the Christoffel symbols spread over the threads. Bound by that chain's latency: the tables of a 24x12x8
+// block, which the no-allocation step forms on every call, took about 90 us more with a thread per point;
+// now 22 us. Every warp also runs the floors' power for a few of its lanes, so a 256x128 plane takes 0.3 ms
+// longer this way: from 6144 points on k_geometry_points.
+constexpr int GEO_T = 12, GEO_P = 8;  // threads per point (eleven places and the floors), points per CTA
 
 __global__ void __launch_bounds__(GEO_T* GEO_P) k_geometry(GeomArgs A) {
     __shared__ double sg[GEO_P][9][7];   // covariant entries: centre, x1 + 2h, + h, - h, - 2h, the same in x2
@@ -84,8 +145,8 @@ __global__ void __launch_bounds__(GEO_T* GEO_P) k_geometry(GeomArgs A) {
     __syncthreads();
     // 4th-order differences of the 7 non-zero entries
     const int pm[7] = {0, 0, 0, 1, 1, 2, 3}, pn[7] = {0, 1, 3, 1, 3, 2, 3};
-    if (on && r < 14) {
-        const int s = r / 7, e = r % 7;
+    for (int c = r; on && c < 14; c += GEO_T) {
+        const int s = c / 7, e = c % 7;
         const double(*g)[7] = &sg[pt][1 + 4 * s];
         const double d = (A.metric != HAMR_METRIC_MINKOWSKI)
                              ? (8.0 * (g[1][e] - g[2][e]) - (g[0][e] - g[3][e])) / (12.0 * CONN_H)
@@ -117,7 +178,10 @@ __global__ void __launch_bounds__(GEO_T* GEO_P) k_geometry(GeomArgs A) {
         }
         n += m;
         double s = 0.0;
-        for (int k = 0; k < 4; k++) s += gi(l, k) * (dg(m, k, n) + dg(n, k, m) - dg(k, m, n));
+        for (int k = 0; k < 4; k++) {
+            const double c_lk = gi(l, k);
+            if (c_lk != 0.0) s += c_lk * (dg(m, k, n) + dg(n, k, m) - dg(k, m, n));
+        }
         A.centre[(C_CONN + c) * n2d + q] = 0.5 * s;
     }
 }
@@ -137,7 +201,10 @@ cudaError_t launch_table_f32(const double* src, float* dst, int nplanes, long st
 
 cudaError_t launch_geometry(const GeomArgs& A, cudaStream_t s) {
     const long n2d = (long)A.n1p * A.n2p;
-    k_geometry<<<(unsigned)((n2d + GEO_P - 1) / GEO_P), GEO_T * GEO_P, 0, s>>>(A);
+    if (n2d >= 6144)
+        k_geometry_points<<<(unsigned)((n2d + 127) / 128), 128, 0, s>>>(A);
+    else
+        k_geometry<<<(unsigned)((n2d + GEO_P - 1) / GEO_P), GEO_T * GEO_P, 0, s>>>(A);
     return cudaGetLastError();
 }
 
