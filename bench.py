@@ -643,6 +643,8 @@ def run_ours(args, rank, world, local):
                     "unit": "TFLOP/s", "frac": achieved / FP64_NOMINAL_TFLOPS,
                     "peak_source": "nominal GB300 FP64 1.25 TFLOP/s (profiling recipe)",
                     "measured_fp64_fma_tflops": fp64_meas, "frac_of_measured": achieved / fp64_meas,
+                    "flops": "algorithmic (the oracle's count); the signal speeds and HLL weights run in "
+                             "double-float on the FP32 pipe, so frac is no utilisation of the FP64 pipe",
                     "traffic": NCU_TRAFFIC_PER_LAUNCH, "avg_launch_ms": dom_ms / launches,
                     "share_of_step": dom_ms / ms}
     whole = FLOPS_PER_ZONE_CYCLE * cells * args.steps / (ms * 1e-3) / 1e12
