@@ -25,8 +25,10 @@ constexpr double C2P_VSQMAX = 1.0 - 1.0 / (50.0 * 50.0);
 enum { INV_OK = 0, INV_ENTROPY = 1, INV_FAIL = 2 };
 
 // how Newton iterates: in double-float with an FP64 last solve (newton_wv_ff), in FP32 with one FP64
-// refinement step (newton_wv_mixed), or in FP64 (newton_wv: grids of the mixed forms, update.cu)
-enum { C2P_NEWTON_FF = 0, C2P_NEWTON32 = 1, C2P_NEWTON64 = 2 };
+// refinement step (newton_wv_mixed), or in FP64 (newton_wv: grids of the mixed forms, update.cu).
+// C2P_NEWTON_ANY: newton_wv_ff from a start that may be anywhere (the standalone inversion), which gives up
+// its double-float iterations early, and the FP64 entropy backup alone
+enum { C2P_NEWTON_FF = 0, C2P_NEWTON32 = 1, C2P_NEWTON64 = 2, C2P_NEWTON_ANY = 3 };
 
 // The normal-frame scalars of a conserved state (Sec. 2.6, Noble et al. 2006).
 struct C2PScalars {
@@ -128,8 +130,13 @@ static __device__ __noinline__ NewtonOut newton_wv_call(const C2PScalars* S, dou
 // An FP64 iteration is ~52 FP64 instructions (64 cycles each per scheduler), here ~340 FP32 ones, plus
 // ~28 FP64 for the solve: 1,000,003 states from a 5% start (4.7 iterations) 1021 -> 626 us, the FP64
 // cell update of the 256x128x64 torus 2.00 -> 1.50 ms with the entropy backup below.
+// any: the start may be far off (no previous state). From such starts many states meet no root, and a warp
+// with one of them waits for 30 iterations in double-float and then for 30 in FP64: a fourth step that still
+// moves the root by a quarter of W ends the first. 1M states at rest (14% without an energy root) take
+// 17.5 ms, 22.0 without the rule, 17.3 with FP64 alone. The cell updates do without it: their failing cells
+// are few, and the cells that get there in more steps would go to FP64 (64x32x16 step 3% slower with it).
 __device__ __forceinline__ bool newton_wv_ff(const C2PScalars& S, double gfac, double& W, double& vsq, int& it,
-                                             double& rs64) {
+                                             double& rs64, bool any) {
     rs64 = 0.0;
     const unsigned eW = (unsigned)__double2hiint(W) & 0xfff00000u;  // sign and exponent of the start
     bool ok = false;
@@ -173,6 +180,7 @@ __device__ __forceinline__ bool newton_wv_ff(const C2PScalars& S, double gfac, d
             cancel = (fabsf(j11.h * j22.h) + fabsf(j12.h * j21.h)) * fabsf(id.h);
             const float tol = (float)C2P_TOL * wn.h, noise = 1e-13f * cancel * wn.h;
             if (noise > 0.5f * tol || (err > 0.25f * before && before < 1e-6f * wn.h)) break;
+            if (any && it >= 4 && err > 0.25f * wn.h) break;
             if (err < tol) {
                 ok = err + noise < tol && before > tol + noise && (err < 1e-3f * before || err < 0.1f * tol);
                 j11h = j11.h;
@@ -427,7 +435,7 @@ struct C2PWork {
     double W0, vsq0;  // the start from the guess primitives
     double p0;        // ... and its pressure (the Aitken inversion's start)
     int method;       // HAMR_INV_NEWTON or HAMR_INV_AITKEN
-    int form;         // Newton: C2P_NEWTON_FF, C2P_NEWTON32 or C2P_NEWTON64
+    int form;         // Newton: C2P_NEWTON_FF, _32, _64 or _ANY
     double igam, gfac;  // 1/gam and (gam - 1)/gam, from one division per inversion
     double W, vsq, rho, u;
     double rs;        // 1/sqrt(1 - v^2) of an energy result
@@ -513,7 +521,7 @@ __device__ __forceinline__ void c2p_attempt(C2PWork& w, double gam, double W, do
     w.rs = 0.0;
     bool ok = (w.form == C2P_NEWTON32)   ? newton_wv_mixed(w.S, gfac, W, vsq, it)
               : (w.form == C2P_NEWTON64) ? newton_wv(w.S, gfac, W, vsq, it)
-                                         : newton_wv_ff(w.S, gfac, W, vsq, it, w.rs);
+                                         : newton_wv_ff(w.S, gfac, W, vsq, it, w.rs, w.form == C2P_NEWTON_ANY);
     w.its += it;
     w.W = W;
     w.vsq = vsq;
@@ -591,7 +599,8 @@ __device__ __forceinline__ void entropy_point(const C2PScalars& S, double gam, d
 // Few cells come here (0.2% of a large torus, 4% of a small one), but their warps wait for this chain:
 // five or six FP64 iterations of ~145 FP64 instructions each before. On a 64x32x16 block the cell update,
 // which such warps end, went from 112 to 67 us (with newton_wv_ff). fast = false: the FP64 iteration alone (the mixed forms,
-// whose results stay bit for bit, update.cu).
+// whose results stay bit for bit, update.cu; the standalone inversion, where many states of a warp may have
+// no entropy root either: 1M inversions by entropy alone, 10% of them failing, 9.41 ms, 9.96 with the FP32 start).
 static __device__ __noinline__ EntropyOut entropy_backup(const C2PScalars* Sp, double kappa, double gam, double W0,
                                                          bool fast) {
     const C2PScalars& S = *Sp;
