@@ -6,8 +6,7 @@
 // warp instruction holds its scheduler's share of the FP64 pipe for 64 cycles,
 // a product below takes 5 issue slots and a sum 11, while that pipe stays free
 // for other work. These numbers stand in where 46 bits change no result: in
-// factors of differences that are small against what they are added to, and
-// in iterations whose last step is taken from FP64 residuals.
+// iterations whose last step is taken from FP64 residuals.
 //
 // Range: that of binary32. Callers scale by powers of two (exact) so that
 // values are O(1); a value below 2^-74 keeps one word, one below 2^-126 is 0.
@@ -71,10 +70,16 @@ __device__ __forceinline__ ff ff_norm(ff a) {
     return ff{h, __fsub_rn(a.l, __fsub_rn(h, a.h))};
 }
 
-// 1 / x: the hardware's approximate reciprocal (2^-23) and one Newton correction in the low word
-__device__ __forceinline__ ff ff_rcp(ff x) {
+// the hardware's approximate reciprocal (2^-23)
+__device__ __forceinline__ float rcp_approx(float x) {
     float r;
-    asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x.h));
+    asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// 1 / x: the approximate reciprocal and one Newton correction in the low word
+__device__ __forceinline__ ff ff_rcp(ff x) {
+    const float r = rcp_approx(x.h);
     float e = __fmaf_rn(-x.h, r, 1.0f);
     e = __fmaf_rn(-x.l, r, e);
     return ff{r, r * e};
@@ -102,6 +107,5 @@ __device__ __forceinline__ ff ff_sqrt_pos(ff x) {
 __device__ __forceinline__ bool ff_less(ff a, ff b) {  // of normalised numbers
     return a.h < b.h || (a.h == b.h && a.l < b.l);
 }
-__device__ __forceinline__ ff ff_max(ff a, ff b) { return ff_less(a, b) ? b : a; }
 
 }  // namespace hamr

@@ -50,8 +50,9 @@ struct BlockView {
 struct PhysArgs {
     double gam;
     double igam, gfac;  // 1/gam and (gam - 1)/gam, formed once on the host
-    float cs2h, cs2l;   // gam (gam - 1) and gam (2 - gam) as sums of two binary32 values: gam p = cs2 u and
-    float wmph, wmpl;   // w - gam p = rho + wmp u of the wave speeds (ff.cuh)
+    double cs2, wmp;    // gam (gam - 1) and gam (2 - gam): gam p = cs2 u and w - gam p = rho + wmp u of the wave speeds
+    float cs2h, cs2l;   // the same as sums of two binary32 values (ff.cuh)
+    float wmph, wmpl;
     double cour;
     int recon;
     int riemann;
@@ -141,11 +142,12 @@ inline void set_gam(PhysArgs& ph, double gam) {
     ph.gam = gam;
     ph.igam = 1.0 / gam;
     ph.gfac = (gam - 1.0) * ph.igam;
-    const double a = gam * (gam - 1.0), b = gam * (2.0 - gam);
-    ph.cs2h = (float)a;
-    ph.cs2l = (float)(a - (double)ph.cs2h);
-    ph.wmph = (float)b;
-    ph.wmpl = (float)(b - (double)ph.wmph);
+    ph.cs2 = gam * (gam - 1.0);
+    ph.wmp = gam * (2.0 - gam);
+    ph.cs2h = (float)ph.cs2;
+    ph.cs2l = (float)(ph.cs2 - (double)ph.cs2h);
+    ph.wmph = (float)ph.wmp;
+    ph.wmpl = (float)(ph.wmp - (double)ph.wmph);
 }
 
 // the launch-shape defaults (what hamr_grid_autotune starts from)

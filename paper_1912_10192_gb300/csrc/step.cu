@@ -568,72 +568,96 @@ __device__ __noinline__ Weights64 hll_weights_fp64(int riemann, double gam, doub
     return w;
 }
 
-// The fast-speed quadratic of one side (wave_quadratic) in double-float; its coefficients scale with
-// (rho, u, b^2), so these enter times a power of two that brings the largest to [1, 2): the speeds
-// (B +- sd)/A do not change.
+// The signal speeds of one side in double-float, from the fast-speed quadratic (wave_quadratic); its
+// coefficients scale with (rho, u, b^2), so these enter times a power of two, 2^(sh >> 20), that brings the
+// largest to [1, 2): the speeds (B +- sd)/A do not change. ok: every factor in binary32's normal range with room
+// for the low words of the squares under the root (NaNs fail too), and the root not lost to cancellation.
 struct WaveFF {
-    ff A, B, sd;
+    ff vp, vm;  // (B +- sd)/A
+    float isd;  // 1/(2 sd), sd = sqrt(B^2 - A C)
+    int sh;
+    bool ok;
 };
 template <int DIR>
 __device__ __forceinline__ WaveFF wave_ff(const PhysArgs& ph, double rho, double u, double bsq, double ut, double ud,
                                           ff c00, ff c0d, ff cdd) {
-    const int sh = scale_of(rho, u, bsq);
-    const ff R = ff_of(rho, sh), U = ff_of(u, sh), b = ff_of(bsq, sh), t = ff_of(ut), d = ff_of(ud);
+    WaveFF w;
+    w.sh = scale_of(rho, u, bsq);
+    const ff R = ff_of(rho, w.sh), U = ff_of(u, w.sh), b = ff_of(bsq, w.sh), t = ff_of(ut), d = ff_of(ud);
     const ff num = ff_add(b, ff_mul(ff{ph.cs2h, ph.cs2l}, U));
     const ff dn = ff_add(R, ff_mul(ff{ph.wmph, ph.wmpl}, U));
     const ff td = ff_mul(t, dn);
-    WaveFF w;
-    w.A = ff_sub(ff_mul(td, t), ff_mul(num, c00));
-    w.B = ff_mul(td, d);
-    if (DIR == 1) w.B = ff_sub(w.B, ff_mul(num, c0d));
+    const ff A = ff_sub(ff_mul(td, t), ff_mul(num, c00));
+    ff B = ff_mul(td, d);
+    if (DIR == 1) B = ff_sub(B, ff_mul(num, c0d));
     const ff C = ff_sub(ff_mul(ff_mul(d, dn), d), ff_mul(num, cdd));
-    w.sd = ff_sqrt_pos(ff_sub(ff_mul(w.B, w.B), ff_mul(w.A, C)));
+    const ff sd = ff_sqrt_pos(ff_sub(ff_mul(B, B), ff_mul(A, C)));
+    const ff iA = ff_rcp(A);
+    w.vp = ff_norm(ff_mul(ff_add(B, sd), iA));
+    w.vm = ff_norm(ff_mul(ff_sub(B, sd), iA));
+    w.isd = 0.5f * rcp_approx(sd.h);
+    w.ok = A.h > 1e-12f && A.h < 1e18f && sd.h > 1e-13f && sd.h < 1e18f && sd.h > 4e-6f * fabsf(B.h);
     return w;
 }
 
-// HLL weights in double-float. wl comes from the ratio of the speeds, wr = sqrt(-g) - wl is its exact
-// complement, so an error in the ratio moves the flux only by itself times F_L - F_R, and one in wc by
-// itself times U_R - U_L: 2^-46 of the jump between the two sides, which in smooth flow is far below the
-// rounding of the fluxes themselves. Speeds as numerators over A_L A_R: Nmax / (Nmax + Nmin) and
-// Nmin / (A_L A_R). false where a number leaves the range (or A <= 0): hll_weights_fp64 then.
+// One Newton step in FP64 on a double-float root x of the fast-speed quadratic A x^2 - 2 B x + C, written as
+// dn (u^t x - u^d)^2 - num (g^tt x^2 - 2 g^td x + g^dd), whose two parts meet at the root without the cancellation
+// of B^2 - A C. hi: 1/(the quadratic's slope) up to its sign, +-1/(2 sd).
+template <int DIR>
+__device__ __forceinline__ double wave_root64(const PhysArgs& ph, double rho, double u, double bsq, double ut,
+                                              double ud, double c00, double c0d, double cdd, ff v, float hi, int sh) {
+    const double x = ff_d(v);
+    const double num = fma(ph.cs2, u, bsq), dn = fma(ph.wmp, u, rho);
+    const double w = fma(ut, x, -ud);
+    const double g = fma((DIR == 1) ? fma(c00, x, -2.0 * c0d) : c00 * x, x, cdd);
+    const double res = fma(dn * w, w, -(num * g));
+    return x + widen(ff_of(res, sh).h * hi);
+}
+
+// HLL weights: the speeds in double-float on the FP32 pipe, the largest and the smallest then taken to FP64 by a
+// Newton step each, the weights in FP64. The double-float speeds alone (2^-46, times the cancellation in
+// B^2 - A C) are not enough: a face between dense and thin gas carries their error into the thin cell as many
+// times larger as the gas is thinner (17x9x16 torus, one step: utilde^2 8e-13 off, 5e-14 with FP64 weights or these).
+// The step leaves what FP64 residuals resolve, no more than the FP64 form's own error, in cold flow less. Which
+// side has the larger speed is decided in double-float, which can err only where the two speeds differ by less
+// than its error. 28 FP64 instructions a face, the FP64 form about 65: a direction of the
+// 256x128x64 torus takes 0.66 ms, 0.55 with the weights left in double-float, a pass of two steps 20.4 ms against
+// 23.0 with the FP64 form. false where a number leaves the range or the root is lost to cancellation:
+// hll_weights_fp64 then.
 template <int DIR>
 __device__ __forceinline__ bool hll_weights_ff(const PhysArgs& ph, const Metric<double>& m, const double pl[NPRIM],
                                                const Side64& sl, const double pr[NPRIM], const Side64& sr,
                                                Weights64& w) {
-    const ff c00 = ff_of(m.c00), c0d = (DIR == 1) ? ff_of(m.c01) : ff{0.0f, 0.0f};
-    const ff cdd = ff_of((DIR == 1) ? m.c11 : ((DIR == 2) ? m.c22 : m.c33));
+    const double cdd = gcondd(m, DIR);
+    const ff c00 = ff_of(m.c00), c0d = (DIR == 1) ? ff_of(m.c01) : ff{0.0f, 0.0f}, cddf = ff_of(cdd);
     const double udl = (DIR == 1) ? sl.u1 : ((DIR == 2) ? sl.u2 : sl.u3);
     const double udr = (DIR == 1) ? sr.u1 : ((DIR == 2) ? sr.u2 : sr.u3);
-    const WaveFF L = wave_ff<DIR>(ph, pl[RHO], pl[UU], sl.bsq, sl.ut, udl, c00, c0d, cdd);
-    const WaveFF R = wave_ff<DIR>(ph, pr[RHO], pr[UU], sr.bsq, sr.ut, udr, c00, c0d, cdd);
-    const ff zero{0.0f, 0.0f};
-    const ff nmax = ff_max(zero, ff_max(ff_norm(ff_mul(ff_add(L.B, L.sd), R.A)), ff_norm(ff_mul(ff_add(R.B, R.sd), L.A))));
-    const ff nmin = ff_max(zero, ff_max(ff_norm(ff_mul(ff_sub(L.sd, L.B), R.A)), ff_norm(ff_mul(ff_sub(R.sd, R.B), L.A))));
-    const ff AA = ff_mul(L.A, R.A), ns = ff_add(nmax, nmin);
-    const ff den = ff_mul(AA, ns);
-    // every factor in the normal range, the squares under the roots (~ ns^2) with room for their low words;
-    // NaNs fail too
-    if (!(L.A.h > 1e-12f && R.A.h > 1e-12f && ns.h > 1e-13f && den.h > 1e-24f && den.h < 1e30f && ns.h < 1e18f &&
-          AA.h < 1e30f))
-        return false;
-    if (nmin.h == 0.0f || nmax.h == 0.0f) {  // both signals leave to one side: that side's flux
-        w.wl = (nmin.h == 0.0f) ? m.gdet : 0.0;
-        w.wr = (nmin.h == 0.0f) ? 0.0 : m.gdet;
-        w.wc = 0.0;
-        return true;
-    }
-    const ff r = ff_rcp(ff_norm(den));
-    w.wl = m.gdet * ff_d(ff_norm(ff_mul(ff_mul(nmax, AA), r)));
-    w.wr = m.gdet - w.wl;
-    w.wc = w.wl * ff_d(ff_norm(ff_mul(ff_mul(nmin, ns), r)));
+    const WaveFF L = wave_ff<DIR>(ph, pl[RHO], pl[UU], sl.bsq, sl.ut, udl, c00, c0d, cddf);
+    const WaveFF R = wave_ff<DIR>(ph, pr[RHO], pr[UU], sr.bsq, sr.ut, udr, c00, c0d, cddf);
+    if (!(L.ok && R.ok)) return false;
+    auto root = [&](bool right, ff v, float hi, int sh) {
+        return wave_root64<DIR>(ph, right ? pr[RHO] : pl[RHO], right ? pr[UU] : pl[UU], right ? sr.bsq : sl.bsq,
+                                right ? sr.ut : sl.ut, right ? udr : udl, m.c00, m.c01, cdd, v, hi, sh);
+    };
+    const bool rp = ff_less(L.vp, R.vp), rm = ff_less(R.vm, L.vm);
+    const double vp = root(rp, rp ? R.vp : L.vp, rp ? -R.isd : -L.isd, rp ? R.sh : L.sh);
+    const double vm = root(rm, rm ? R.vm : L.vm, rm ? R.isd : L.isd, rm ? R.sh : L.sh);
+    const double cmax = max_i(0.0, vp), cmin = max_i(0.0, -vm), sum = cmax + cmin;
+    const float s32 = ff_of(sum).h;
+    if (!(s32 > 1e-18f && s32 < 1e18f)) return false;
+    const double y = widen(rcp_approx(s32)), e = fma(-sum, y, 1.0);  // 1/sum = y (1 + e + e^2 + ...), |e| < 2^-21
+    const double r = m.gdet * fma(y, fma(e, e, e), y);
+    w.wl = cmax * r;
+    w.wr = cmin * r;
+    w.wc = cmax * w.wr;
     return true;
 }
 
 // HLLE (or LLF) flux in FP64 through every dir-face: faces 0..n_dir, -1..n_e across. Bound by the FP64
 // pipe (2 lanes per SM and cycle), so what counts is FP64 instructions per face: the side states
-// without b^mu and b_mu, and the weights (about 65 of the former 220) moved to the idle FP32 pipe.
-// 256x128x64 torus, one direction: 0.857 ms with the FP64 weights and lowered b^mu, 0.554 ms now; the
-// error of a step against a 64-bit reference is unchanged (1.4e-14).
+// without b^mu and b_mu, and the weights (28 of the former 65 or so) started on the idle FP32 pipe.
+// 256x128x64 torus, one direction: 0.857 ms with the FP64 weights and lowered b^mu, 0.66 ms now; the
+// error of a step against 80-bit arithmetic is that of FP64 throughout.
 template <int DIR>
 __device__ __forceinline__ void b_flux64(const BlockView& v, const PhysArgs& ph, const double* __restrict__ QL,
                                          const double* __restrict__ QR, const double* __restrict__ Bf,
