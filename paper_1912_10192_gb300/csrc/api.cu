@@ -1,8 +1,10 @@
 // api.cu -- the C ABI declared in include/hamr.h: grid lifetime, state I/O,
 // the per-block midpoint step and the standalone inversion.
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <cmath>
+#include <cstdint>
 #include <cstdarg>
 #include <cstdio>
 #include <algorithm>
@@ -29,10 +31,14 @@ int fail(int code, const char* fmt, ...) {
     return code;
 }
 
-#define CUDA_TRY(call)                                                                                   \
-    do {                                                                                                 \
-        cudaError_t e_ = (call);                                                                         \
-        if (e_ != cudaSuccess) return fail(HAMR_ECUDA, "%s failed: %s", #call, cudaGetErrorString(e_)); \
+// a failed call's error is the caller's: it does not stay behind for the next launch's check
+#define CUDA_TRY(call)                                                                            \
+    do {                                                                                          \
+        cudaError_t e_ = (call);                                                                  \
+        if (e_ != cudaSuccess) {                                                                  \
+            cudaGetLastError();                                                                   \
+            return fail(HAMR_ECUDA, "%s failed: %s", #call, cudaGetErrorString(e_));              \
+        }                                                                                         \
     } while (0)
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -374,16 +380,35 @@ int copy_fields(double* dst, long dstride, const double* src, long sstride, long
     return HAMR_OK;
 }
 
-// Whether a kernel on the grid's device can take the pointer: memory of that device, or managed. Other
-// pointers (another device's, page-locked or plain host memory) go through the runtime's copies, which take
-// what they can and refuse the rest.
-bool kernel_can_reach(const hamr_grid* g, const void* p) {
+// Whether a kernel on the grid's device can take `bytes` bytes of doubles at p: aligned, in memory of that device
+// or managed, within one allocation. Everything else (another device's, page-locked or plain host memory, a
+// pointer into the middle of a value, a range past its allocation or over several mappings) goes through the
+// runtime's copies, which take what they can and refuse the rest with an error.
+bool kernel_can_reach(const hamr_grid* g, const void* p, size_t bytes) {
+    if ((uintptr_t)p % alignof(double) != 0) return false;
     cudaPointerAttributes a;
     if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
-    return (a.type == cudaMemoryTypeDevice && a.device == g->device) || a.type == cudaMemoryTypeManaged;
+    if (!((a.type == cudaMemoryTypeDevice && a.device == g->device) || a.type == cudaMemoryTypeManaged)) return false;
+    using Query = CUresult (*)(unsigned, CUpointer_attribute*, void**, CUdeviceptr);
+    static const Query query = [] {  // the driver's query, found at run time (no link against libcuda)
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult r;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault, &r) != cudaSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return (Query)f;
+    }();
+    CUpointer_attribute which[2] = {CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    CUdeviceptr start = 0;
+    size_t size = 0;
+    void* out[2] = {&start, &size};
+    if (!query || query(2, which, out, (CUdeviceptr)p) != CUDA_SUCCESS) return false;
+    const size_t at = (size_t)((CUdeviceptr)p - start);
+    return (CUdeviceptr)p >= start && at <= size && bytes <= size - at;
 }
 
 int check_block(const hamr_grid* g, int block) {
@@ -475,7 +500,8 @@ int hamr_grid_set_state(hamr_grid* g, int block, const double* prim, const doubl
     const BlockView& v = g->view[block];
     BlockState& s = g->st[block];
     const long n = (long)v.n1p * v.n2p * v.n3p;
-    if (on_device && kernel_can_reach(g, prim) && kernel_can_reach(g, bface)) {
+    const size_t field = sizeof(double) * (size_t)n;
+    if (on_device && kernel_can_reach(g, prim, 8 * field) && kernel_can_reach(g, bface, 3 * field)) {
         cudaStream_t cs = S(stream);
         double *Po = nullptr, *Bo = nullptr;
         if (g->amr) amr_old_state(g->amr, block, &Po, &Bo);  // no history yet: the previous state is the loaded one
@@ -511,7 +537,11 @@ int hamr_grid_get_state(const hamr_grid* g, int block, double* prim, double* bfa
     const BlockView& v = g->view[block];
     const BlockState& s = g->st[block];
     const long n = (long)v.n1p * v.n2p * v.n3p;
-    if (on_device && (prim || bface) && (!prim || kernel_can_reach(g, prim)) && (!bface || kernel_can_reach(g, bface))) {
+    const size_t field = sizeof(double) * (size_t)n;
+    const uintptr_t pa = (uintptr_t)prim, ba = (uintptr_t)bface;
+    const bool apart = !prim || !bface || pa + 8 * field <= ba || ba + 3 * field <= pa;  // else the copies' order counts
+    if (on_device && (prim || bface) && apart && (!prim || kernel_can_reach(g, prim, 8 * field)) &&
+        (!bface || kernel_can_reach(g, bface, 3 * field))) {
         CUDA_TRY(launch_store(v, s.P, s.B, prim, bface, S(stream)));
         return HAMR_OK;
     }
