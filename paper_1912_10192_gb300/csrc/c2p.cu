@@ -57,8 +57,9 @@ __global__ void __launch_bounds__(128) k_con2prim(hamr_c2p_desc d, const uint8_t
             }
         }
     }
+    if (active && !entropy_only && !(MLP && rescue)) c2p_attempt_plain(w, d.gam);
+    __syncwarp();  // the lanes come out of the attempt by several ways: together again for the backup
     if (!active) return;
-    if (!entropy_only && !(MLP && rescue)) c2p_attempt_plain(w, d.gam);
     const int st = c2p_finish(w, u, m, d.gam, pr);
     const int it = w.its;
 #pragma unroll

@@ -128,13 +128,16 @@ static __device__ __noinline__ NewtonOut newton_wv_call(const C2PScalars* S, dou
 // double-float iteration meets no root or leaves its range, newton_wv decides. `it` counts the iterations,
 // not the solve. rs: 1/sqrt(1 - v^2) at the root where it comes for free, else 0.
 // An FP64 iteration is ~52 FP64 instructions (64 cycles each per scheduler), here ~340 FP32 ones, plus
-// ~28 FP64 for the solve: 1,000,003 states from a 5% start (4.7 iterations) 1021 -> 626 us, the FP64
+// ~28 FP64 for the solve: 1M states from a 5% start (4.7 iterations) 1035 -> 626 us, the FP64
 // cell update of the 256x128x64 torus 2.00 -> 1.50 ms with the entropy backup below.
 // any: the start may be far off (no previous state). From such starts many states meet no root, and a warp
 // with one of them waits for 30 iterations in double-float and then for 30 in FP64: a fourth step that still
 // moves the root by a quarter of W ends the first. 1M states at rest (14% without an energy root) take
-// 17.5 ms, 22.0 without the rule, 17.3 with FP64 alone. The cell updates do without it: their failing cells
-// are few, and the cells that get there in more steps would go to FP64 (64x32x16 step 3% slower with it).
+// 12.7 ms, 16.8 without the rule, 12.0 with FP64 alone; 30 to 50% off 8.1, 6.9 and 7.9 ms. The cell updates do
+// without it: their failing cells are few, and cells that get there in more steps would go to FP64.
+// Lanes leave by several ways (root taken, FP64 after each of the breaks, early break there), and the compiler
+// brings them together as late as it may: callers put a __syncwarp() behind the attempt, without which the
+// entropy backup ran once for each way (1M states at rest 17.5 ms).
 __device__ __forceinline__ bool newton_wv_ff(const C2PScalars& S, double gfac, double& W, double& vsq, int& it,
                                              double& rs64, bool any) {
     rs64 = 0.0;
@@ -598,9 +601,10 @@ __device__ __forceinline__ void entropy_point(const C2PScalars& S, double gam, d
 // meets no root, or the second FP64 step is not below the rule, the FP64 iteration runs from the start.
 // Few cells come here (0.2% of a large torus, 4% of a small one), but their warps wait for this chain:
 // five or six FP64 iterations of ~145 FP64 instructions each before. On a 64x32x16 block the cell update,
-// which such warps end, went from 112 to 67 us (with newton_wv_ff). fast = false: the FP64 iteration alone (the mixed forms,
-// whose results stay bit for bit, update.cu; the standalone inversion, where many states of a warp may have
-// no entropy root either: 1M inversions by entropy alone, 10% of them failing, 9.41 ms, 9.96 with the FP32 start).
+// which such warps end, takes 49 us a launch, 98 with FP64 iterations alone (newton_wv's too). fast = false:
+// the FP64 iteration alone, in the mixed forms, whose results stay bit for bit (update.cu), and in the
+// standalone inversion, where many states of a warp may have no entropy root either (1M inversions by
+// entropy alone, 10% of them failing: 9.41 ms, 9.96 with the FP32 start).
 static __device__ __noinline__ EntropyOut entropy_backup(const C2PScalars* Sp, double kappa, double gam, double W0,
                                                          bool fast) {
     const C2PScalars& S = *Sp;

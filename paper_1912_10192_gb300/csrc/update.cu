@@ -121,6 +121,11 @@ __device__ __forceinline__ void b_update64(const BlockView& v, const PhysArgs& p
     if (active) {
         c2p_prepare(U, Bc, m, gam, pr, w, ph.inversion, C2P_NEWTON_FF, nullptr, ph.igam, ph.gfac, start);
         c2p_attempt_plain(w, gam);
+    }
+    // the lanes come out of the attempt by several ways: together again, or the entropy backup runs once for
+    // each (pair of launches on a 24x12x8 block 207 -> 120 us, 96x64x48 disk with MINMOD 1180 -> 720 us)
+    __syncwarp();
+    if (active) {
         its = w.its;
         st = c2p_finish(w, U, m, gam, pr);
         uint8_t sb = (st == INV_ENTROPY) ? ST_ENTROPY : ((st == INV_FAIL) ? ST_FAIL : 0);
@@ -263,8 +268,9 @@ __device__ __forceinline__ void b_update(const BlockView& v, const PhysArgs& ph,
         c2p_prepare(U, Bc, m, gam, pr, w, ph.inversion, INV64 ? C2P_NEWTON64 : C2P_NEWTON32,
                     have32 ? start32 : nullptr, ph.igam, ph.gfac);
     if (MLP) mlp_attempts(C, mlp_smem, ph, rescue, active, w, U, m, v.x1min + (i + 0.5) * v.dx1);
+    if (active && !rescue) c2p_attempt_plain(w, gam);
+    __syncwarp();  // as in b_update64 (24x12x8 pair, mixed: 225 -> 185 us)
     if (active) {
-        if (!rescue) c2p_attempt_plain(w, gam);
         its = w.its;
         st = c2p_finish(w, U, m, gam, pr);
         uint8_t sb = (st == INV_ENTROPY) ? ST_ENTROPY : ((st == INV_FAIL) ? ST_FAIL : 0);
