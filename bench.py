@@ -47,10 +47,12 @@ FLOPS_PER_ZONE_CYCLE = 4605.0    # one cell, one full step
 # Peaks. FP64: nominal GB300 rate (the profiling recipe's 1.25 TFLOP/s); the
 # FMA rate measured by hamr_measure_fp64_peak is reported beside it.
 FP64_NOMINAL_TFLOPS = 1.25
-# DRAM bytes per launch of the dominant kernel group, from one ncu capture
-# of this build's x1-face flux kernel (the x2 and x3 kernels move the same
-# field sizes): 312.5 MB read + 115.4 MB written.
-NCU_TRAFFIC_PER_LAUNCH = 427.9e6
+# Instructions on the FP64 pipe per unit of work (mean over the launches of one
+# step) and DRAM bytes per launch of the x1-face flux kernel (the x2 and x3 ones
+# move the same field sizes; 311.8 MB read + 115.7 MB written), from the ncu
+# capture in profiles/fp64_kernels_torus256.md.
+FP64_INSTR = {"flux": 169.1, "recon": 100.7, "update": 323.6}
+NCU_TRAFFIC_PER_LAUNCH = 427.5e6
 
 
 def env_rank():
@@ -631,20 +633,18 @@ def run_ours(args, rank, world, local):
     name, (launches, dom_ms) = dom
     steps = args.steps
     faces = ((N1 + 1) * (N2 + 2) * (N3 + 2) + (N1 + 2) * (N2 + 1) * (N3 + 2) + (N1 + 2) * (N2 + 2) * (N3 + 1))
-    per_step_units = {"flux": FLOPS_PER_FACE * faces * 2,
-                      "recon": FLOPS_PER_RECON_CELL * 3 * (N1 + 2) * (N2 + 2) * (N3 + 2) * 2,
-                      "update": FLOPS_PER_UPDATE_CELL * cells * 2}
+    per_step_units = {"flux": faces * 2, "recon": 3 * (N1 + 2) * (N2 + 2) * (N3 + 2) * 2, "update": cells * 2}
+    per_unit = {"flux": FLOPS_PER_FACE, "recon": FLOPS_PER_RECON_CELL, "update": FLOPS_PER_UPDATE_CELL}
     roofline = None
     if name in per_step_units:
-        flops_per_launch = per_step_units[name] * steps / launches
-        avg_s = dom_ms * 1e-3 / launches
-        achieved = flops_per_launch / avg_s / 1e12
+        units = per_step_units[name] * steps / (dom_ms * 1e-3)  # per second
+        achieved = 2.0 * FP64_INSTR[name] * units / 1e12
         roofline = {"bound": "alu", "kernel": name, "achieved": achieved, "peak": FP64_NOMINAL_TFLOPS,
                     "unit": "TFLOP/s", "frac": achieved / FP64_NOMINAL_TFLOPS,
                     "peak_source": "nominal GB300 FP64 1.25 TFLOP/s (profiling recipe)",
                     "measured_fp64_fma_tflops": fp64_meas, "frac_of_measured": achieved / fp64_meas,
-                    "flops": "algorithmic (the oracle's count); the signal speeds and HLL weights run in "
-                             "double-float on the FP32 pipe, so frac is no utilisation of the FP64 pipe",
+                    "flops": "instructions on the FP64 pipe (ncu), two operations each: frac is that pipe's use",
+                    "algorithmic_tflops": per_unit[name] * units / 1e12,
                     "traffic": NCU_TRAFFIC_PER_LAUNCH, "avg_launch_ms": dom_ms / launches,
                     "share_of_step": dom_ms / ms}
     whole = FLOPS_PER_ZONE_CYCLE * cells * args.steps / (ms * 1e-3) / 1e12

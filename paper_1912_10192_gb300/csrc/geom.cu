@@ -101,9 +101,10 @@ __global__ void k_geometry_points(GeomArgs A) {
 // centre, four around it in x1 and four in x2 for the derivatives, the two faces), each a chain of FP64
 // transcendental functions: one place per thread, the covariant entries shared through shared memory, then
 // the Christoffel symbols spread over the threads. Bound by that chain's latency: the tables of a 24x12x8
-// block, which the no-allocation step forms on every call, took about 90 us more with a thread per point;
-// now 22 us. Every warp also runs the floors' power for a few of its lanes, so a 256x128 plane takes 0.3 ms
-// longer this way: from 6144 points on k_geometry_points.
+// block, which the no-allocation step forms on every call, take 20 us, 57 with a thread per point, which takes
+// that long up to 15000 points. Every warp also runs the floors' power for a few of its lanes, so the time
+// here grows with the points: 43 us at 4000, 62 at 6144, 295 at 35108 (256x128; 108 with a thread per point).
+// The two meet between: from 6144 points on k_geometry_points.
 constexpr int GEO_T = 12, GEO_P = 8;  // threads per point (eleven places and the floors), points per CTA
 
 __global__ void __launch_bounds__(GEO_T* GEO_P) k_geometry(GeomArgs A) {

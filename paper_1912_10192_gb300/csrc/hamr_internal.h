@@ -112,7 +112,9 @@ constexpr int RECON_TILE = 28;
 constexpr int RECON_SEG = 16;  // default sweep length
 constexpr int RECON_X1_SWEEP = 1;  // default form of the x1 edge values
 // FP32: cells per thread along dir for a launch over this many cells (4, along x1 2, where that leaves 8 warps
-// or so per scheduler of the 152 SMs, b_recon_cells)
+// or so per scheduler of the 152 SMs, b_recon_cells). x1 + x2 + x3, one cell per thread against groups: 18 and
+// 28 us at 43142 cells, 21 and 28 at 131072, 35 and 34 at 270336, 71 and 67 at 589824, 115 and 97 at 1048576,
+// 220 and 183 at 2097152: the line is safe rather than sharp, below it the groups gain at most a tenth
 inline int recon_cells(long cells, int dir) { return cells < 152L * 4 * 8 * 32 * 4 ? 1 : (dir == 1 ? 2 : 4); }
 __host__ __device__ inline long recon_threads(const BlockView& v, int dir, int m, int seg, int x1_sweep = 0) {
     const long n1 = v.n1 + 2, n2 = v.n2 + 2, n3 = v.n3 + 2;

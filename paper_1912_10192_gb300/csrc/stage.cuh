@@ -108,7 +108,6 @@ __device__ __forceinline__ double inv_dt_cell(const BlockView& v, const T pr[NPR
     return inv_dt_fluid(v, pr, s, m, gam);
 }
 
-// the rate of a cell in precision T from its (FP64) primitives
 // source sqrt(-g) T^k_l Gamma^l_{nu k} at a cell centre in precision T
 // (tables gc: metric and connection planes of that precision)
 template <typename T, typename TT>

@@ -1,9 +1,10 @@
 // step.cu -- the per-block stage kernels of the midpoint step
 // (Liska et al. 2019, Sec. 2.1 and 2.5-2.7).
 //
-// One stage = boundary conditions (3 passes) -> per direction: edge values
+// One stage = boundary conditions (one launch) -> per direction: edge values
 // (reconstruction) and face fluxes -> edge EMFs -> CT face update ->
-// cell update + inversion + floors (+ CFL reduction in the corrector).
+// cell update + inversion + floors (+ CFL reduction in the corrector), the
+// last in update.cu.
 // Fluxes, EMFs and edge values go through HBM: the FP64 path is bound by the
 // FP64 pipe, so every face flux and every parabola is computed exactly once
 // and re-read from memory instead of recomputed in a halo.
@@ -617,10 +618,10 @@ __device__ __forceinline__ double wave_root64(const PhysArgs& ph, double rho, do
 // HLL weights: the speeds in double-float on the FP32 pipe, the largest and the smallest then taken to FP64 by a
 // Newton step each, the weights in FP64. The double-float speeds alone (2^-46, times the cancellation in
 // B^2 - A C) are not enough: a face between dense and thin gas carries their error into the thin cell as many
-// times larger as the gas is thinner (17x9x16 torus, one step: utilde^2 8e-13 off, 5e-14 with FP64 weights or these).
+// times larger as the gas is thinner (17x9x16 torus, one step: utilde^2 8e-13 off, 5e-14 with FP64 weights, 6e-14 here).
 // The step leaves what FP64 residuals resolve, no more than the FP64 form's own error, in cold flow less. Which
 // side has the larger speed is decided in double-float, which can err only where the two speeds differ by less
-// than its error. 28 FP64 instructions a face, the FP64 form about 65: a direction of the
+// than its error. About 30 FP64 instructions of the 170 a face takes, the FP64 form about 65: a direction of the
 // 256x128x64 torus takes 0.66 ms, 0.55 with the weights left in double-float, a pass of two steps 20.4 ms against
 // 23.0 with the FP64 form. false where a number leaves the range or the root is lost to cancellation:
 // hll_weights_fp64 then.
@@ -655,7 +656,7 @@ __device__ __forceinline__ bool hll_weights_ff(const PhysArgs& ph, const Metric<
 
 // HLLE (or LLF) flux in FP64 through every dir-face: faces 0..n_dir, -1..n_e across. Bound by the FP64
 // pipe (2 lanes per SM and cycle), so what counts is FP64 instructions per face: the side states
-// without b^mu and b_mu, and the weights (28 of the former 65 or so) started on the idle FP32 pipe.
+// without b^mu and b_mu, and the weights (30 of the former 65 or so) started on the idle FP32 pipe.
 // 256x128x64 torus, one direction: 0.857 ms with the FP64 weights and lowered b^mu, 0.66 ms now; the
 // error of a step against 80-bit arithmetic is that of FP64 throughout.
 template <int DIR>
@@ -707,10 +708,11 @@ __device__ __forceinline__ void b_flux64(const BlockView& v, const PhysArgs& ph,
 }
 
 // HLLE (or LLF) flux in FP32 (mixed precision).
-template <int DIR, typename T>
-__device__ __forceinline__ void b_flux32(const BlockView& v, PhysArgs ph, const T* __restrict__ QL,
-                                             const T* __restrict__ QR, const double* __restrict__ Bf,
-                                             double* __restrict__ F, long t) {
+template <int DIR>
+__device__ __forceinline__ void b_flux32(const BlockView& v, const PhysArgs& ph, const float* __restrict__ QL,
+                                         const float* __restrict__ QR, const double* __restrict__ Bf,
+                                         double* __restrict__ F, long t) {
+    using T = float;
     const int nn[4] = {0, v.n1, v.n2, v.n3};
     const int e1 = (DIR == 1) ? nn[1] + 1 : nn[1] + 2;
     const int e2 = (DIR == 2) ? nn[2] + 1 : nn[2] + 2;
@@ -724,7 +726,7 @@ __device__ __forceinline__ void b_flux32(const BlockView& v, PhysArgs ph, const 
     Metric<T> m;
     load_metric(face_table<DIR, T>(v), v.n2d, gidx(v, i, j), m);
     // single-block mixed precision: the two field slots (6, 7) also in FP32, after the FP64 fields
-    float* F32 = (std::is_same<T, float>::value && ph.flux32) ? reinterpret_cast<float*>(F + NFLUX * v.nc) : nullptr;
+    float* F32 = ph.flux32 ? reinterpret_cast<float*>(F + NFLUX * v.nc) : nullptr;
     if (m.gdet == T(0)) {  // face on the polar axis: no area
 #pragma unroll
         for (int q = 0; q < NFLUX; q++) F[q * v.nc + c] = 0.0;
@@ -781,8 +783,8 @@ __device__ __forceinline__ void b_flux32(const BlockView& v, PhysArgs ph, const 
 #pragma unroll
     for (int q = 0; q < NFLUX; q++) F[q * v.nc + c] = (double)acc[q];
     if (F32) {
-        F32[c] = (float)acc[6];
-        F32[v.nc + c] = (float)acc[7];
+        F32[c] = acc[6];
+        F32[v.nc + c] = acc[7];
     }
 }
 
@@ -793,7 +795,7 @@ __device__ __forceinline__ void b_flux(const BlockView& v, const PhysArgs& ph, c
     if constexpr (std::is_same<T, double>::value)
         b_flux64<DIR>(v, ph, QL, QR, Bf, F, t);
     else
-        b_flux32<DIR, T>(v, ph, QL, QR, Bf, F, t);
+        b_flux32<DIR>(v, ph, QL, QR, Bf, F, t);
 }
 
 template <int DIR, typename T>

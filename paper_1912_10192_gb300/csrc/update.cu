@@ -8,9 +8,14 @@
 // where a value sits at a rounding boundary a change of its last bit moves that stage
 // by an FP32 unit, which limiters and the inversion of magnetised cells then amplify
 // (measured with the same arithmetic in double-float, 2^-46: one cell in 3000 off by
-// more than 1e-8 after four steps). With the network attached a start's last bit
-// decides in the same way which root a failing cell is rescued to, so FP64 keeps the
-// same form there.
+// more than 1e-8 after four steps). FP64 cells under the network keep Newton in FP64:
+// with newton_wv_ff a test of tree periods gave other outcomes from run to run (cells
+// whose rescue by the network sits on a knife edge: a change of the last bit of rho and
+// u moves a tilted disk's step by 1e-2 in either form). They keep the rest of b_update
+// with it only because no FP64 form with the network has been made from b_update64: a
+// step of the 256x128x64 torus takes 13.1 / 12.3 ms with the network first / as rescue,
+// 10.0 without. Inversions in which the network has no part (internal-SMR groups,
+// refluxed cells, drift-frame floors) take the same form on every FP64 grid.
 #include "mlp.cuh"
 #include "stage.cuh"
 
@@ -329,7 +334,7 @@ __global__ void __launch_bounds__(BS) k_update64(BlockView v, PhysArgs ph, HAMR_
     b_update64<COR>(v, ph, true, Pf, F1, F2, F3, Bn, Un, Po, status, dscal, fac, dmax, dcnt, tidx());
 }
 // four CTAs per SM (128 registers, a few spilled) without the network: the FP64 pipe waits less between the
-// FP32 stretches (256x128x64 torus, mixed: 0.96 -> 0.92 ms per launch; 384 threads per CTA: 1.09 ms)
+// FP32 stretches (256x128x64 torus, mixed predictor: 1.03 -> 0.94 ms; 384 threads per CTA: 1.09 ms)
 template <bool MLP, typename TS, bool INV64>
 __global__ void __launch_bounds__(BS, MLP ? 3 : 4) k_update(BlockView v, PhysArgs ph, int corrector, HAMR_UPD_PARAMS) {
     b_update<MLP, TS, INV64>(v, ph, corrector, Pf, F1, F2, F3, Bn, Un, Po, status, dscal, fac, dmax, dcnt, tidx());
