@@ -20,10 +20,11 @@ constexpr int TSMP = 64;  // samples per CTA of the training kernel
 constexpr int TTHR = 256; // its threads
 constexpr int HS = 68;    // row stride of its 64-wide arrays: 16-byte aligned rows, 16 bytes apart modulo the banks
 constexpr int XS = 12;    // row stride of its 10-wide arrays (two zeros)
-// shared memory of k_mlp_fb (floats): W2, W3, three hidden layers, W1, inputs, biases and W4, output errors
+// shared memory of k_mlp_fb (floats): W2, W3, three hidden layers, W1, inputs, biases and W4, output errors,
+// four warps' sums of squares
 constexpr int FB_W2 = 0, FB_W3 = 64 * HS, FB_H1 = 2 * 64 * HS, FB_H2 = FB_H1 + TSMP * HS, FB_H3 = FB_H2 + TSMP * HS,
               FB_W1 = FB_H3 + TSMP * HS, FB_X = FB_W1 + 64 * XS, FB_B = FB_X + TSMP * XS, FB_W4 = FB_B + 192,
-              FB_B4 = FB_W4 + 128, FB_DY = FB_B4 + 4, FB_N = FB_DY + TSMP * 2;
+              FB_B4 = FB_W4 + 128, FB_DY = FB_B4 + 4, FB_R2 = FB_DY + TSMP * 2, FB_N = FB_R2 + 4;
 constexpr int FB_SMEM = FB_N * 4;
 
 __device__ __forceinline__ uint64_t splitmix64(uint64_t x) {  // Steele, Lea & Flood (2014)
@@ -197,7 +198,7 @@ __global__ void __launch_bounds__(TTHR) k_mlp_fb(const float* __restrict__ Pg, c
                                                  int64_t step, float* __restrict__ grad, float* __restrict__ loss) {
     extern __shared__ __align__(16) float fsm[];
     float *W2 = fsm + FB_W2, *W3 = fsm + FB_W3, *H1 = fsm + FB_H1, *H2 = fsm + FB_H2, *H3 = fsm + FB_H3;
-    float *W1 = fsm + FB_W1, *X = fsm + FB_X, *Bs = fsm + FB_B, *W4 = fsm + FB_W4, *B4 = fsm + FB_B4, *DY = fsm + FB_DY;
+    float *W1 = fsm + FB_W1, *X = fsm + FB_X, *Bs = fsm + FB_B, *W4 = fsm + FB_W4, *B4 = fsm + FB_B4, *DY = fsm + FB_DY, *R2 = fsm + FB_R2;
     const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
     auto sample = [&](int s, int64_t& g) {  // whether sample s of the CTA counts, and its row
         const int64_t b = (int64_t)blockIdx.x * TSMP + s;
@@ -242,7 +243,6 @@ __global__ void __launch_bounds__(TTHR) k_mlp_fb(const float* __restrict__ Pg, c
     __syncthreads();
     mlp_layer<64, HS>(H2, W3, Bs + 128, H3, tx, ty);
     __syncthreads();
-    float r2 = 0.0f;
     if (t < 2 * TSMP) {
         const int s = t >> 1, j = t & 1;
         int64_t g;
@@ -257,8 +257,10 @@ __global__ void __launch_bounds__(TTHR) k_mlp_fb(const float* __restrict__ Pg, c
             y = fmaf(w.w, h.w, y);
         }
         const float r = on ? y - (targ[j * n + g] - norm[20 + j]) / norm[22 + j] : 0.0f;
-        r2 = r * r;
         DY[s * 2 + j] = r * (1.0f / (float)count);
+        float v = r * r;
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if ((t & 31) == 0) R2[t >> 5] = v;
     }
     __syncthreads();
     // output layer gradients: (j, o) over half the samples each
@@ -365,10 +367,8 @@ __global__ void __launch_bounds__(TTHR) k_mlp_fb(const float* __restrict__ Pg, c
             if (i0 + q < MLP_NIN) atomicAdd(&grad[P_W1 + o * MLP_NIN + i0 + q], acc[q]);
         if ((t & 3) == 0) atomicAdd(&grad[P_B1 + o], bs);
     }
-    // loss
-    float v = r2;
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((t & 31) == 0 && t < 2 * TSMP) atomicAdd(loss, v);
+    // loss: one sum per CTA, as the running sum's rounding grows with the number of its terms
+    if (t == 0) atomicAdd(loss, (R2[0] + R2[1]) + (R2[2] + R2[3]));
 }
 
 __global__ void k_adam(float* __restrict__ P, float* __restrict__ grad, float* __restrict__ m1,
