@@ -355,7 +355,8 @@ int hamr_block_step_noalloc(const hamr_grid_desc* d, double* prim, double* bface
 /* ---- standalone inversion (Sec. 2.6) ----
  * Without HAMR_C2P_MIXED or HAMR_C2P_AITKEN: Newton in double-float that ends
  * with a solve of the FP64 residuals, in FP64 from starts that are far off or
- * ill-conditioned; the entropy backup in FP64. */
+ * ill-conditioned and in batches of up to 128 states per SM; the entropy
+ * backup in FP64. */
 #define HAMR_C2P_ENTROPY_ONLY 1u /* skip the energy inversion (tests of the backup) */
 #define HAMR_C2P_MLP 2u          /* start Newton from the learned guess of `mlp` (fallback: the prim guess) */
 #define HAMR_C2P_MLP_RESCUE 4u   /* start from the prim guess; where that fails, from the learned guess */

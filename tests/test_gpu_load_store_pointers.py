@@ -68,3 +68,23 @@ def test_short_allocation_is_refused():
     assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1])
     g.close()
     assert cu.cuMemFree_v2(ptr) == 0
+
+
+def test_under_capture():
+    """A load and a read-out captured into a graph, with the pointers asked about during the capture."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    g, (prim, bf) = _grid_and_state()
+    p, b = torch.from_numpy(prim).cuda(), torch.from_numpy(bf).cuda()
+    po, bo = torch.zeros_like(p), torch.zeros_like(b)
+    g.set_state(p, b)
+    want = g.get_state()
+    s, gr = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(gr, stream=s):
+        g.set_state(p, b, stream=s)
+        g.get_state(prim=po, bface=bo, stream=s)
+    gr.replay()
+    torch.cuda.synchronize()
+    assert np.array_equal(po.cpu().numpy(), want[0]) and np.array_equal(bo.cpu().numpy(), want[1])
+    g.close()
